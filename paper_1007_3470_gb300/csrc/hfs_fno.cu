@@ -11,6 +11,7 @@
 
 #include "hfs.h"
 #include "hfs_fno.h"
+#include "hfs_fno_fused.h"
 #include "hfs_fno_kernels.cuh"
 #include "hfs_fno_tc.cuh"
 
@@ -248,6 +249,66 @@ int refresh_weights(hfs_fno_s *f)
     to_bf16_kernel<<<blocks(C * P), 256, 0, st>>>(f->params + f->po.P1, at<bf16>(f, f->off.P1b), C * P);
     to_bf16_kernel<<<blocks(P * c.out_ch), 256, 0, st>>>(f->params + f->po.P2, at<bf16>(f, f->off.P2b), P * c.out_ch);
     FCK(cudaGetLastError());
+    return HFS_OK;
+}
+
+FusedDims fused_dims(const hfs_fno_s *f)
+{
+    const hfs_fno_config &c = f->cfg;
+    return {c.grid, c.width, c.modes, c.proj, c.in_ch, c.out_ch, c.layers, f->max_batch};
+}
+
+// the sizes that the fused kernels are built for take them; the rest, and the
+// tcgen05 engine, go GEMM by GEMM (forward below)
+bool use_fused(const hfs_fno_s *f) { return f->gemm_engine == HFS_FNO_GEMM_MMA_SYNC && fused_ok(fused_dims(f)); }
+
+// the forward pass, a stage kernel before, between and after the layers'
+// mixing products; train: the activations that the backward pass reads are kept
+int forward_fused(hfs_fno_s *f, const float *x, int B, float *out, bool train)
+{
+    const int64_t C = f->cfg.width, M = f->cfg.modes, NL = f->cfg.layers, Bm = f->max_batch;
+    const int64_t rowsM = Bm * f->cfg.grid;
+    cudaStream_t st = f->stream;
+    const auto &w = f->off;
+    StageArgs a{};
+    a.d = fused_dims(f);
+    a.B = B;
+    a.x = x;
+    a.Pinb = at<bf16>(f, w.Pinb);
+    a.bin = f->params + f->po.bin;
+    a.F2 = at<bf16>(f, w.F2);
+    a.Gre = at<bf16>(f, w.Gre);
+    a.Gim = at<bf16>(f, w.Gim);
+    a.Y = at<bf16>(f, w.Yb);
+    bf16 *Hb = at<bf16>(f, w.Hb);
+    // S of every layer is kept when training
+    auto S = [&](int64_t l) { return at<bf16>(f, w.S) + (train ? l * Bm * 2 * M * C : 0); };
+    StageArgs first = a;
+    first.S = S(0);
+    first.Hout = train ? Hb : nullptr;
+    FCK(launch_stage(first, true, false, false, false, st));
+    for (int64_t l = 0; l < NL; ++l) {
+        FCK(launch_mix(a.d, B, S(l), at<bf16>(f, w.Rb1) + l * M * C * 2 * C, at<bf16>(f, w.Rb2) + l * M * C * 2 * C,
+                       at<bf16>(f, w.Yb), st));
+        StageArgs s = a;
+        s.Hin = Hb + l * rowsM * C;
+        s.W = at<bf16>(f, w.Wb) + l * C * C;
+        s.bias = f->params + f->po.b[l];
+        s.pre = train ? at<float>(f, w.pre) + l * rowsM * C : nullptr;
+        const bool head = l == NL - 1;
+        s.Hout = (train || !head) ? Hb + (l + 1) * rowsM * C : nullptr;
+        if (head) {
+            s.P1b = at<bf16>(f, w.P1b);
+            s.c1 = f->params + f->po.c1;
+            s.P2b = at<bf16>(f, w.P2b);
+            s.c2 = f->params + f->po.c2;
+            s.Qpre = train ? at<float>(f, w.Qpre) : nullptr;
+            s.O = out;
+        } else {
+            s.S = S(l + 1);
+        }
+        FCK(launch_stage(s, l == 0, true, head, true, st));
+    }
     return HFS_OK;
 }
 
@@ -588,6 +649,7 @@ int hfs_fno_forward(hfs_fno_t f, const float *x, float *y, int32_t batch)
     if (!f->params || !f->work) return HFS_ERR_NOT_READY;
     if (batch < 1 || batch > f->max_batch) return HFS_ERR_INVALID_ARG;
     (void)cudaGetLastError();
+    if (use_fused(f)) return forward_fused(f, x, batch, y, false);
     int s = forward(f, x, batch);
     if (s) return s;
     FCK(cudaMemcpyAsync(y, at<float>(f, f->off.O), 4 * (size_t)batch * f->cfg.grid * f->cfg.out_ch,

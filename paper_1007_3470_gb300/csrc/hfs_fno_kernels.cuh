@@ -3,13 +3,10 @@
 // epilogues, and the elementwise, reduction, loss and Adam kernels around it.
 #pragma once
 
-#include <cuda_bf16.h>
-#include <stdint.h>
+#include "hfs_fno_frag.cuh"
 
 namespace hfs {
 namespace fno {
-
-typedef __nv_bfloat16 bf16;
 
 // C[b] = alpha * op(A[b]) op(B[b]) (+ beta C[b]) (+ bias[n]) (+ add[b]) -> [pre] -> GELU? -> C, Cb
 //   op(A)(m, k) = TA ? A[k lda + m] : A[m lda + k]
@@ -37,33 +34,6 @@ struct GemmArgs {
 };
 
 constexpr int GT_M = 64, GT_N = 64, GT_K = 32, GT_LD = 40;  // smem rows padded to 40 bf16 (80 B)
-
-__device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad_f(float z)
-{
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
-}
-
-__device__ __forceinline__ void ldsm_x4(unsigned (&r)[4], const bf16 *p)
-{
-    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(a));
-}
-__device__ __forceinline__ void ldsm_x2(unsigned (&r)[2], const bf16 *p)
-{
-    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(a));
-}
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4], const unsigned (&b)[2])
-{
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
 
 // Load a ROWS x 32 (k) tile into smem as [row][k], from a matrix whose rows
 // (m or n) are either k-contiguous (KCONT) or row-contiguous (the transposed
@@ -180,25 +150,6 @@ template <bool TA, bool TB> __global__ void __launch_bounds__(128) gemm_bf16_ker
 // multiples of 8 (gemm_pipe_ok).
 // ---------------------------------------------------------------------------
 constexpr int GP_STAGES = 3, GP_LDT = 72;  // transposed tiles: [32 k][64 + 8]
-
-__device__ __forceinline__ void ldsm_x4_t(unsigned (&r)[4], const bf16 *p)
-{
-    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(a));
-}
-__device__ __forceinline__ void ldsm_x2_t(unsigned (&r)[2], const bf16 *p)
-{
-    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(a));
-}
-// 16-byte asynchronous copy; an invalid chunk is zero-filled (source size 0)
-__device__ __forceinline__ void cp16(bf16 *dst, const bf16 *src, bool valid)
-{
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(valid ? 16 : 0) : "memory");
-}
 
 inline bool gemm_pipe_ok(const GemmArgs &g, bool ta, bool tb)
 {
