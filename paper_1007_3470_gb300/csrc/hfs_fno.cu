@@ -230,25 +230,40 @@ cudaError_t weight_grad(int M, int N, int64_t rows, const bf16 *A, int64_t lda, 
     return run(g, true, false, st);
 }
 
-int refresh_weights(hfs_fno_s *f)
+RefreshArgs refresh_args(hfs_fno_s *f)
 {
     const hfs_fno_config &c = f->cfg;
-    const int64_t C = c.width, M = c.modes, P = c.proj;
-    cudaStream_t st = f->stream;
-    to_bf16_pad_kernel<<<blocks((int64_t)kInPad * C), 256, 0, st>>>(f->params + f->po.Pin, c.in_ch, (int)C,
-                                                                     at<bf16>(f, f->off.Pinb), (int)C);
+    RefreshArgs r{};
+    r.n = f->nparams;
+    r.bin = f->po.bin;
+    r.layer0 = f->po.Rre[0];
+    r.layer_stride = (f->po.P1 - f->po.Rre[0]) / c.layers;
+    r.P1 = f->po.P1;
+    r.c1 = f->po.c1;
+    r.P2 = f->po.P2;
+    r.c2 = f->po.c2;
+    r.in_ch = c.in_ch;
+    r.C = c.width;
+    r.M = c.modes;
+    r.P = c.proj;
+    r.out_ch = c.out_ch;
+    r.p = f->params;
+    r.Pinb = at<bf16>(f, f->off.Pinb);
+    r.Wb = at<bf16>(f, f->off.Wb);
+    r.R1 = at<bf16>(f, f->off.Rb1);
+    r.R2 = at<bf16>(f, f->off.Rb2);
+    r.P1b = at<bf16>(f, f->off.P1b);
+    r.P2b = at<bf16>(f, f->off.P2b);
+    return r;
+}
+
+int refresh_weights(hfs_fno_s *f)
+{
     // P_in is [in_ch][C]: pad rows in_ch..7 with zeros
-    if (c.in_ch < kInPad)
-        FCK(cudaMemsetAsync(at<bf16>(f, f->off.Pinb) + (int64_t)c.in_ch * C, 0, 2 * (kInPad - c.in_ch) * C, st));
-    for (int l = 0; l < c.layers; ++l) {
-        to_bf16_kernel<<<blocks(C * C), 256, 0, st>>>(f->params + f->po.W[l], at<bf16>(f, f->off.Wb) + l * C * C, C * C);
-        mixing_weights_kernel<<<blocks(M * C * 2 * C), 256, 0, st>>>(
-            f->params + f->po.Rre[l], f->params + f->po.Rim[l], (int)M, (int)C,
-            at<bf16>(f, f->off.Rb1) + l * M * C * 2 * C, at<bf16>(f, f->off.Rb2) + l * M * C * 2 * C);
-    }
-    to_bf16_kernel<<<blocks(C * P), 256, 0, st>>>(f->params + f->po.P1, at<bf16>(f, f->off.P1b), C * P);
-    to_bf16_kernel<<<blocks(P * c.out_ch), 256, 0, st>>>(f->params + f->po.P2, at<bf16>(f, f->off.P2b), P * c.out_ch);
-    FCK(cudaGetLastError());
+    const int64_t C = f->cfg.width, used = (int64_t)f->cfg.in_ch * C;
+    if (f->cfg.in_ch < kInPad)
+        FCK(cudaMemsetAsync(at<bf16>(f, f->off.Pinb) + used, 0, 2 * (kInPad * C - used), f->stream));
+    FCK(launch_refresh(refresh_args(f), nullptr, f->stream));
     return HFS_OK;
 }
 
@@ -264,7 +279,7 @@ bool use_fused(const hfs_fno_s *f) { return f->gemm_engine == HFS_FNO_GEMM_MMA_S
 
 // the forward pass, a stage kernel before, between and after the layers'
 // mixing products; train: the activations that the backward pass reads are kept
-int forward_fused(hfs_fno_s *f, const float *x, int B, float *out, bool train)
+int forward_fused(hfs_fno_s *f, const float *x, int B, float *out, const float *y, bool train)
 {
     const int64_t C = f->cfg.width, M = f->cfg.modes, NL = f->cfg.layers, Bm = f->max_batch;
     const int64_t rowsM = Bm * f->cfg.grid;
@@ -304,11 +319,68 @@ int forward_fused(hfs_fno_s *f, const float *x, int B, float *out, bool train)
             s.c2 = f->params + f->po.c2;
             s.Qpre = train ? at<float>(f, w.Qpre) : nullptr;
             s.O = out;
+            s.y = y;
+            s.sums = y ? at<float>(f, w.sums) : nullptr;
         } else {
             s.S = S(l + 1);
         }
         FCK(launch_stage(s, l == 0, true, head, true, st));
     }
+    return HFS_OK;
+}
+
+// gradients of the loss after forward_fused with the same targets
+int backward_fused(hfs_fno_s *f, const float *x, const float *y, int B, float *grad)
+{
+    const int64_t C = f->cfg.width, M = f->cfg.modes, NL = f->cfg.layers, Bm = f->max_batch;
+    const int64_t rowsM = Bm * f->cfg.grid;
+    cudaStream_t st = f->stream;
+    const auto &w = f->off;
+    const bf16 *Hb = at<bf16>(f, w.Hb);
+    HeadBwdArgs h{};
+    h.d = fused_dims(f);
+    h.B = B;
+    h.O = at<float>(f, w.O);
+    h.y = y;
+    h.sums = at<float>(f, w.sums);
+    h.Qpre = at<float>(f, w.Qpre);
+    h.H = Hb + NL * rowsM * C;
+    h.P1b = at<bf16>(f, w.P1b);
+    h.P2b = at<bf16>(f, w.P2b);
+    h.dZ = at<bf16>(f, w.dZb);
+    h.gP1 = grad + f->po.P1;
+    h.gc1 = grad + f->po.c1;
+    h.gP2 = grad + f->po.P2;
+    h.gc2 = grad + f->po.c2;
+    h.gb = grad + f->po.b[NL - 1];
+    FCK(launch_head_bwd(h, st));
+    LayerBwdArgs a{};
+    a.d = h.d;
+    a.B = B;
+    a.dZ = h.dZ;
+    a.dSup = at<bf16>(f, w.dSb);
+    a.F2 = at<bf16>(f, w.F2);
+    a.Gre = at<bf16>(f, w.Gre);
+    a.Gim = at<bf16>(f, w.Gim);
+    a.dY = at<bf16>(f, w.dYb);
+    for (int64_t l = NL - 1; l >= 0; --l) {
+        a.Wup = l < NL - 1 ? at<bf16>(f, w.Wb) + (l + 1) * C * C : nullptr;
+        a.pre = at<float>(f, w.pre) + l * rowsM * C;
+        a.Hin = Hb + l * rowsM * C;
+        a.gW = grad + f->po.W[l];
+        a.gb = grad + f->po.b[l];
+        FCK(launch_layer_bwd(a, l == NL - 1 ? LayerBwd::kTop : LayerBwd::kMid, st));
+        FCK(launch_mix_bwd(a.d, B, at<bf16>(f, w.S) + l * Bm * 2 * M * C, at<bf16>(f, w.dYb),
+                           at<bf16>(f, w.Rb1) + l * M * C * 2 * C, at<bf16>(f, w.Rb2) + l * M * C * 2 * C,
+                           at<bf16>(f, w.dSb), grad + f->po.Rre[l], grad + f->po.Rim[l], st));
+    }
+    a.Wup = at<bf16>(f, w.Wb);
+    a.x = x;
+    a.gW = grad + f->po.Pin;
+    a.gb = grad + f->po.bin;
+    FCK(launch_layer_bwd(a, LayerBwd::kLift, st));
+    loss_value_kernel<<<1, 256, 0, st>>>(at<float>(f, w.sums), B, at<float>(f, w.loss));
+    FCK(cudaGetLastError());
     return HFS_OK;
 }
 
@@ -649,7 +721,7 @@ int hfs_fno_forward(hfs_fno_t f, const float *x, float *y, int32_t batch)
     if (!f->params || !f->work) return HFS_ERR_NOT_READY;
     if (batch < 1 || batch > f->max_batch) return HFS_ERR_INVALID_ARG;
     (void)cudaGetLastError();
-    if (use_fused(f)) return forward_fused(f, x, batch, y, false);
+    if (use_fused(f)) return forward_fused(f, x, batch, y, nullptr, false);
     int s = forward(f, x, batch);
     if (s) return s;
     FCK(cudaMemcpyAsync(y, at<float>(f, f->off.O), 4 * (size_t)batch * f->cfg.grid * f->cfg.out_ch,
@@ -663,10 +735,16 @@ int hfs_fno_loss_grad(hfs_fno_t f, const float *x, const float *y, int32_t batch
     if (!f->params || !f->work || !f->train) return HFS_ERR_NOT_READY;
     if (batch < 1 || batch > f->max_batch) return HFS_ERR_INVALID_ARG;
     (void)cudaGetLastError();
-    int s = forward(f, x, batch);
-    if (s) return s;
     float *g = grad ? grad : at<float>(f, f->off.grad);
-    s = backward(f, y, batch, g);
+    int s;
+    if (use_fused(f) && fused_train_ok(fused_dims(f))) {
+        FCK(cudaMemsetAsync(g, 0, 4 * f->nparams, f->stream));
+        s = forward_fused(f, x, batch, at<float>(f, f->off.O), y, true);
+        if (!s) s = backward_fused(f, x, y, batch, g);
+    } else {
+        s = forward(f, x, batch);
+        if (!s) s = backward(f, y, batch, g);
+    }
     if (s) return s;
     if (loss_host) {
         FCK(cudaMemcpyAsync(loss_host, at<float>(f, f->off.loss), 4, cudaMemcpyDeviceToHost, f->stream));
@@ -682,12 +760,9 @@ int hfs_fno_train_step(hfs_fno_t f, const float *x, const float *y, int32_t batc
     f->step += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - powf(b1, (float)f->step), c2 = 1.0f - powf(b2, (float)f->step);
-    adam_kernel<<<blocks(f->nparams), 256, 0, f->stream>>>(f->params, at<float>(f, f->off.grad),
-                                                            at<float>(f, f->off.m), at<float>(f, f->off.v),
-                                                            f->nparams, lr, b1, b2, 1e-8f, c1, c2);
-    FCK(cudaGetLastError());
-    s = refresh_weights(f);
-    if (s) return s;
+    const AdamArgs adam{at<float>(f, f->off.grad), at<float>(f, f->off.m), at<float>(f, f->off.v), lr, b1, b2, 1e-8f,
+                        c1, c2};
+    FCK(launch_refresh(refresh_args(f), &adam, f->stream));
     if (loss_host) {
         FCK(cudaMemcpyAsync(loss_host, at<float>(f, f->off.loss), 4, cudaMemcpyDeviceToHost, f->stream));
         FCK(cudaStreamSynchronize(f->stream));

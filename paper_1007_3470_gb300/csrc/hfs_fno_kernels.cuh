@@ -324,12 +324,6 @@ __global__ void to_bf16_pad_kernel(const float *x, int64_t rows, int cin, bf16 *
     out[i] = __float2bfloat16(c < cin ? x[r * cin + c] : 0.0f);
 }
 
-__global__ void to_bf16_kernel(const float *x, bf16 *out, int64_t n)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) out[i] = __float2bfloat16(x[i]);
-}
-
 // dZ = dH * gelu'(pre) (or dH when apply == 0); FP32 and BF16 outputs
 __global__ void gelu_bwd_kernel(const float *dH, const float *pre, int apply, float *dZ, bf16 *dZb, int64_t n)
 {
@@ -405,33 +399,6 @@ __global__ void loss_value_kernel(const float *sums, int batch, float *loss)
         __syncthreads();
     }
     if (threadIdx.x == 0) *loss = red[0] / (float)batch;
-}
-
-__global__ void adam_kernel(float *p, const float *g, float *m, float *v, int64_t n, float lr, float b1, float b2,
-                            float eps, float c1, float c2)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
-
-// complex mixing weights as real blocks: R1[k] = [Rre | Rim], R2[k] = [-Rim | Rre] ([C][2C])
-__global__ void mixing_weights_kernel(const float *Rre, const float *Rim, int M, int C, bf16 *R1, bf16 *R2)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= (int64_t)M * C * 2 * C) return;
-    const int64_t k = i / (C * 2 * C);
-    const int64_t r = (i / (2 * C)) % C;
-    const int col = (int)(i % (2 * C));
-    const int64_t src = (k * C + r) * C + (col % C);
-    const float re = Rre[src], im = Rim[src];
-    R1[i] = __float2bfloat16(col < C ? re : im);
-    R2[i] = __float2bfloat16(col < C ? -im : re);
 }
 
 // gradients of Rre, Rim from those of R1, R2

@@ -53,3 +53,56 @@ def test_forward_does_not_depend_on_the_batch(batch):
     whole = m.forward(x)
     assert torch.equal(whole, torch.cat([m.forward(p) for p in x.split(17)]))
     m.close()
+
+
+@pytest.mark.parametrize("cfg", CONFIGS)
+@pytest.mark.parametrize("batch", [1, 31])
+def test_gradients_equal_gemm_by_gemm(cfg, batch):
+    """Loss and gradients: the same rounded operands, FP32 sums in another
+    order.  A sum of n terms in FP32 differs between two orders by at most
+    n 2^-24 of the sum of its terms' magnitudes and by sqrt(n) 2^-24 of their
+    root mean square as a rule; with n = 8192 rows at most that is 5.4e-6 of a
+    gradient's norm, and a BF16 rounding that falls the other way moves one
+    operand in thousands by 2^-8 (about 3e-5 of a norm together)."""
+    torch = need_gpu()
+    from paper_1007_3470_gb300.fno import HFS_FNO_GEMM_TCGEN05
+    m, x, y = _model(cfg, batch)
+    loss, g = m.loss_grad(x, y)
+    m.set_gemm_engine(HFS_FNO_GEMM_TCGEN05)
+    loss_ref, ref = m.loss_grad(x, y)
+    assert abs(loss - loss_ref) <= 1e-6 * loss_ref
+    assert torch.isfinite(ref).all()
+    assert float((g - ref).norm()) <= 5e-5 * float(ref.norm())
+    m.close()
+
+
+def test_gradient_vector_need_not_be_aligned():
+    """A gradient vector on a 4-byte boundary that is no 8-byte boundary."""
+    torch = need_gpu()
+    import ctypes
+    from paper_1007_3470_gb300.fno import _lib
+    m, x, y = _model(CONFIGS[1], 5)
+    _, ref = m.loss_grad(x, y)
+    buf = torch.zeros(m.nparams + 1, device="cuda")
+    torch.cuda.synchronize()
+    vp = ctypes.c_void_p
+    assert _lib().hfs_fno_loss_grad(m.h, vp(x.data_ptr()), vp(y.data_ptr()), 5, vp(buf.data_ptr() + 4), None) == 0
+    m.stream.synchronize()
+    assert float((buf[1:] - ref).norm()) <= 1e-6 * float(ref.norm())
+    m.close()
+
+
+def test_training_steps_follow_the_gemm_by_gemm_path():
+    """Adam and the BF16 weight copies: the losses of a short training run on
+    either path (steps of 1e-3 on weights near 0.2: a gradient entry whose sign
+    is noise moves one weight, the loss by less than 1e-3 of itself)."""
+    need_gpu()
+    from paper_1007_3470_gb300.fno import HFS_FNO_GEMM_TCGEN05
+    losses = []
+    for engine in (0, HFS_FNO_GEMM_TCGEN05):
+        m, x, y = _model(CONFIGS[2], 9)
+        m.set_gemm_engine(engine)
+        losses.append([m.train_step(x, y, 1e-3) for _ in range(12)])
+        m.close()
+    assert losses[0][-1] < losses[0][0]
+    assert np.allclose(losses[0], losses[1], rtol=1e-3)
