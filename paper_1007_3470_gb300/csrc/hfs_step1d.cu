@@ -137,9 +137,8 @@ __global__ void twiddle_plain_kernel(float2 *tp)
 // ---------------------------------------------------------------------------
 size_t step1d_smem_bytes(bool fp64)
 {
-    if (fp64) return (size_t)step1d_exchange_elems * sizeof(cpx<double>);
-    return (size_t)step1d_exchange_elems * sizeof(cpx<float>) +
-           (size_t)(step1d_vtable_floats + step1d_slot_floats) * sizeof(float);
+    const size_t r = fp64 ? sizeof(double) : sizeof(float);
+    return ((size_t)2 * step1d_exchange_elems + step1d_vtable_elems) * r + step1d_slot_floats * sizeof(float);
 }
 
 static cudaError_t prepare_diag(bool fp64)

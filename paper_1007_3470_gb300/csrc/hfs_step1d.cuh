@@ -146,6 +146,18 @@ __device__ __forceinline__ void vi_table(float *vt, int t, const TeamParams<floa
     }
 }
 
+// FP64: cos (about 45 FP64 instructions) once per work item, not per sub-stage
+template <int N, int E, int VI>
+__device__ __forceinline__ void vi_table(double *vt, int t, const TeamParams<double> &tp)
+{
+    constexpr int T = N / E;
+#pragma unroll 1
+    for (int e = 0; e < E; ++e) {
+        const double x = fma((double)(t + T * e - N / 2), tp.dx, tp.xc);
+        vt[t + T * e] = tp.eps * vi_eval(tp.vikind, x, tp.vik);
+    }
+}
+
 // VI >= 0: every instance of the launch has the perturbation kind VI and a
 // box symmetric about 0 (compile-time, no per-point tests); VI = -1: both
 // read from the team's instance.  Run-time tests inside the unrolled loop
@@ -188,22 +200,24 @@ __device__ __forceinline__ void xphase(cpx<float> (&v)[E], int t, const RecF &rc
     }
 }
 
+// FP64: the products enter one sum, rounded once at the size of the largest
+// (as the reduced product of each was), and apply_turns reduces it
 template <int N, int E, int VI>
 __device__ __forceinline__ void xphase(cpx<double> (&v)[E], int t, const RecD &rc, const TeamParams<double> &tp,
-                                       const float *, float &)
+                                       const double *vt, double &)
 {
     constexpr int T = N / E;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
+        if (e % PHASE_GROUP == 0) {
+            fence_group(v, e);
+            asm volatile("" : "+r"(t));
+        }
         const int m = t + T * e - N / 2;
-        const double mf = (double)m;
-        double turns = frac_turns(mf * mf, rc.k2, 0.0);
-        if (tp.asym) turns += frac_turns(mf, rc.k1, 0.0) + rc.k0;
-        const double x = fma(mf, tp.dx, tp.xc);
-        const double dens = v[e].x * v[e].x + v[e].y * v[e].y;
-        const double F = fma(tp.sigma, dens, tp.eps * vi_eval(tp.vikind, x, tp.vik));
-        turns = fma(rc.sb2pi, F, turns);
-        v[e] = apply_turns(v[e], turns, 1.0);
+        const double dens = fma(v[e].x, v[e].x, v[e].y * v[e].y);
+        double turns = rc.sb2pi * fma(tp.sigma, dens, vt[t + T * e]);
+        if (tp.asym) turns += fma(rc.k1, (double)m, rc.k0);
+        v[e] = apply_turns(v[e], fma(rc.k2, square64(m), turns), 1.0);
     }
 }
 
@@ -235,18 +249,21 @@ __device__ __forceinline__ void kphase(cpx<double> (&v)[E], int t, const RecD &r
     constexpr int T = N / E;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        const int k = t + T * e;
-        const double m = (double)((k < N / 2) ? k : k - N);
-        const double turns = frac_turns(m * m, rc.g, 0.0);
-        v[e] = apply_turns(v[e], turns, 1.0 / N);
+        if (e % PHASE_GROUP == 0) {
+            fence_group(v, e);
+            asm volatile("" : "+r"(t));
+        }
+        // |m| of k = t + T e, which is below N/2 where e < E/2
+        const int m = t + T * e - (2 * e < E ? 0 : N);
+        v[e] = apply_turns(v[e], rc.g * square64(m), 1.0 / N);
     }
 }
 
 // complex elements of the exchange buffers of a CTA (the largest over the
-// plans: E = 16 values per thread), and floats of the eps V_I table and of
+// plans: E = 16 values per thread), entries of the eps V_I table and floats of
 // the per-warp norm sums after them
 constexpr int step1d_exchange_elems = (kCtaThreads / (4096 / 16)) * smem_elems(4096);
-constexpr int step1d_vtable_floats = kCtaThreads * 16;
+constexpr int step1d_vtable_elems = kCtaThreads * 16;
 constexpr int step1d_slot_floats = kCtaThreads / 32;
 
 // Norm projection (FP32 path).  The exact scheme is unitary: every sub-flow
@@ -302,7 +319,7 @@ __device__ __forceinline__ void fft(const Step1DArgs &a, cpx<R> (&v)[E], cpx<R> 
 template <typename R, int VI, int N, int E, bool ALT, bool PROJ, typename Rec>
 __device__ __forceinline__ void step_loop(const Step1DArgs &a, cpx<R> (&v)[E], int t, int g, bool active, int idx,
                                           const Rec *rec, const TeamParams<R> &tp, cpx<R> *sm,
-                                          const typename TwOf<R>::type *tw, const float *vt, float *slots)
+                                          const typename TwOf<R>::type *tw, const R *vt, float *slots)
 {
     constexpr int T = N / E;
     // the team's target sum of |u|^2: read, or set from the first sub-stage
@@ -318,7 +335,7 @@ __device__ __forceinline__ void step_loop(const Step1DArgs &a, cpx<R> (&v)[E], i
         // across the whole time loop.
         int tl = t;
         asm volatile("" : "+r"(tl));
-        float dsum = 0.0f;
+        R dsum = 0;
         xphase<N, E, VI>(v, tl, rc, tp, vt, dsum);
         if constexpr (PROJ) dsum = team_sum_begin<T>(dsum, slots);
         fft<false, PROJ, N, ALT>(a, v, sm, tl, tw, g);
@@ -375,6 +392,11 @@ __device__ __forceinline__ void step_item(const Step1DArgs &a, const WorkItem &i
     const int g = threadIdx.x / T;
     const int t = threadIdx.x - g * T;
     const bool active = g < it.count;
+    // a warp without an instance leaves the FP32 and FP64 pipes to the others
+    // (one FP64 instance of 1024 points took 201 us a sub-stage with the three
+    // idle teams of its CTA transforming zeros and the longer phases, 63 us
+    // without; one FP32 instance of 256 points 2.7 us a step, 1.9 us without)
+    if ((threadIdx.x & ~31) / T >= it.count) return;
     const int idx = a.order[it.first + (active ? g : 0)];
     const DevInst &ip = a.inst[idx];
     const TeamParams<R> tp = team_params<R>(ip);
@@ -386,15 +408,15 @@ __device__ __forceinline__ void step_item(const Step1DArgs &a, const WorkItem &i
     cpx<R> v[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = active ? ld_state(psi + t + T * e, a.streaming) : cpx<R>{R(0), R(0)};
-    // FP32: the table of eps V_I behind the exchange buffers (each thread
-    // reads back only the entries it wrote), then the norm-sum slots
-    float *vt = reinterpret_cast<float *>(smem + step1d_exchange_elems) + g * N;
-    float *slots = reinterpret_cast<float *>(smem + step1d_exchange_elems) + step1d_vtable_floats;
-    if constexpr (sizeof(R) == 4 && VI != HFS_VI_NONE) vi_table<N, E, VI>(vt, t, tp);
+    // the table of eps V_I behind the exchange buffers (each thread reads back
+    // only the entries it wrote), then the norm-sum slots
+    R *vt = reinterpret_cast<R *>(smem + step1d_exchange_elems) + g * N;
+    float *slots = reinterpret_cast<float *>(reinterpret_cast<R *>(smem + step1d_exchange_elems) + step1d_vtable_elems);
+    if constexpr (VI != HFS_VI_NONE) vi_table<N, E, VI>(vt, t, tp);
     step_loop<R, VI, N, E, ALT, PROJ && sizeof(R) == 4>(a, v, t, g, active, idx, rec, tp, sm, tw, vt, slots);
     if (a.final_x) {
         const Rec rc = rec[a.j1];
-        float dsum = 0.0f;
+        R dsum = 0;
         xphase<N, E, VI>(v, t, rc, tp, vt, dsum);
     }
     if (active) {

@@ -58,6 +58,16 @@ __global__ void __launch_bounds__(kCtaThreads) xpass3d(const Step3DArgs a, int64
     cpx<R> *sm = reinterpret_cast<cpx<R> *>(smem_raw) + g * smem_elems(N);
     cpx<R> *psi = reinterpret_cast<cpx<R> *>(a.psi) + (int64_t)line * N;
     const auto *tw = reinterpret_cast<const typename TwOf<R>::type *>(a.tw);
+    // V_I along each axis, once per CTA: cos in FP64 costs as much as all other
+    // phase arithmetic of a point
+    __shared__ R s_v[3][N];
+    if constexpr (MODE & X_PHASE) {
+        const DevInst &ip = *a.inst;
+        const int vkind = (ip.eps != 0.0) ? ip.vi_kind : HFS_VI_NONE;
+        for (int i = threadIdx.x; i < 3 * N; i += kCtaThreads)
+            s_v[i / N][i % N] = vi_eval(vkind, (R)(i % N - N / 2) * (R)ip.dx[i / N], (R)ip.vi_k);
+        __syncthreads();
+    }
     cpx<R> v[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = psi[t + T * e];
@@ -65,18 +75,21 @@ __global__ void __launch_bounds__(kCtaThreads) xpass3d(const Step3DArgs a, int64
     if constexpr (MODE & X_PHASE) {
         const Rec rc = reinterpret_cast<const Rec *>(a.rec)[j];
         const DevInst &ip = *a.inst;
-        const int my = y - N / 2, mz = z - N / 2;
-        const R tyz = turns_q(my, rc.k2[1], rc.k2lo[1]) + turns_q(mz, rc.k2[2], rc.k2lo[2]);
-        const R dx = (R)ip.dx[0], vk = (R)ip.vi_k, eps = (R)ip.eps, sig = (R)ip.sigma;
-        const int vkind = (ip.eps != 0.0) ? ip.vi_kind : HFS_VI_NONE;
-        const R vyz = vi_eval(vkind, (R)my * (R)ip.dx[1], vk) + vi_eval(vkind, (R)mz * (R)ip.dx[2], vk);
+        const R tyz = turns_q(y - N / 2, rc.k2[1], rc.k2lo[1]) + turns_q(z - N / 2, rc.k2[2], rc.k2lo[2]);
+        const R eps = (R)ip.eps, sig = (R)ip.sigma;
+        const R vyz = s_v[1][y] + s_v[2][z];
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int mx = t + T * e - N / 2;
-            R turns = turns_q(mx, rc.k2[0], rc.k2lo[0]) + tyz;
             const R dens = v[e].x * v[e].x + v[e].y * v[e].y;
-            const R F = sig * dens + eps * (vi_eval(vkind, (R)mx * dx, vk) + vyz);
-            turns += (R)rc.sb2pi * F;
+            const R F = sig * dens + eps * (s_v[0][mx + N / 2] + vyz);
+            R turns;
+            if constexpr (sizeof(R) == 8) {
+                turns = fma(rc.k2[0], square64(mx), fma((R)rc.sb2pi, F, tyz));
+            } else {
+                turns = turns_q(mx, rc.k2[0], rc.k2lo[0]) + tyz;
+                turns += (R)rc.sb2pi * F;
+            }
             v[e] = apply_turns(v[e], turns, R(1));
         }
     }
@@ -207,7 +220,7 @@ __global__ void __launch_bounds__(kCtaThreads, ZpassMinCtas<R>::value) zpass3d(c
             for (int e = 0; e < E; ++e) {
                 const int kz = t + T * e;
                 const int mz = (kz < N / 2) ? kz : kz - N;
-                v[e] = apply_turns(v[e], txy + turns_q(mz, rc.g[2], rc.glo[2]), scale);
+                v[e] = apply_turns(v[e], fma(rc.g[2], square64(mz), txy), scale);
             }
         }
     }
