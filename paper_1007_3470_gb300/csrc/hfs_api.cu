@@ -854,7 +854,8 @@ int hfs_step(hfs_ctx_t c, int64_t nsteps)
     return HFS_OK;
 }
 
-static int run_diag(hfs_ctx_s *c)
+// norms or energies into diag_host (3D forms both)
+static int run_diag(hfs_ctx_s *c, bool energy)
 {
     (void)cudaGetLastError();
     const bool fp64 = c->precision == HFS_C128;
@@ -869,10 +870,8 @@ static int run_diag(hfs_ctx_s *c)
         a.tw = fp64 ? wptr<void>(c, c->lay.twd) : wptr<void>(c, c->lay.twf);
         a.t_dev = wptr<double>(c, c->lay.tdev);
         a.out = dout;
-        a.ticket = wptr<unsigned>(c, c->lay.ticket);
-        CK(cudaMemsetAsync(a.ticket, 0, sizeof(unsigned), c->stream));
-        const int grid = std::max(1, std::min<int>(a.nwork, c->sm_count * step1d_ctas_per_sm(fp64, c->variant)));
-        CK(launch_diag1d(fp64, a, grid, c->stream));
+        a.pre = wptr<StageFGE>(c, c->lay.fge);  // free between calls
+        CK(launch_diag1d(fp64, energy, a, c->sm_count, c->stream));
     } else {
         Diag3DArgs a{};
         a.psi = c->psi;
@@ -894,7 +893,7 @@ int hfs_norm(hfs_ctx_t c, double *out)
     int s = ready(c);
     if (s) return s;
     if (!out) return HFS_ERR_INVALID_ARG;
-    s = run_diag(c);
+    s = run_diag(c, false);
     if (s) return s;
     for (int64_t i = 0; i < c->count; ++i) out[i] = c->diag_host[2 * i];
     return HFS_OK;
@@ -906,7 +905,7 @@ int hfs_energy(hfs_ctx_t c, double *out)
     int s = ready(c);
     if (s) return s;
     if (!out) return HFS_ERR_INVALID_ARG;
-    s = run_diag(c);
+    s = run_diag(c, true);
     if (s) return s;
     for (int64_t i = 0; i < c->count; ++i) out[i] = c->diag_host[2 * i + 1];
     return HFS_OK;

@@ -153,6 +153,7 @@ __host__ __device__ constexpr int size_class(int n)
 constexpr int kPlanCodes = 4;
 __host__ __device__ constexpr int plan_code(int ept, bool alt) { return ept == 16 ? (alt ? 2 : 0) : ept == 8 ? 1 : 3; }
 __host__ __device__ constexpr int plan_id(int n, int ept, bool alt = false) { return size_class(n) * kPlanCodes + plan_code(ept, alt); }
+__host__ __device__ constexpr int plan_ept(int plan) { return plan % kPlanCodes == 1 ? 8 : plan % kPlanCodes == 3 ? 4 : 16; }
 // codes 2 and 3 live in the "wide" step kernels only (the default kernels
 // keep the smaller instruction footprint)
 __host__ __device__ constexpr bool plan_is_wide(int plan) { return (plan % kPlanCodes) >= 2; }

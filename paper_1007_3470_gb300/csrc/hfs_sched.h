@@ -84,10 +84,11 @@ struct Diag1DArgs {
     int32_t nwork;
     const void *tw;
     const double *t_dev;
-    double *out;  // [count][2]: norm, energy
-    unsigned *ticket;
+    double *out;    // [count][2]: norm, energy
+    StageFGE *pre;  // energy: scratch, one record per instance
 };
-cudaError_t launch_diag1d(bool fp64, const Diag1DArgs &a, int grid, cudaStream_t st);
+// the energies (energy) or the norms of the batch
+cudaError_t launch_diag1d(bool fp64, bool energy, const Diag1DArgs &a, int sms, cudaStream_t st);
 
 cudaError_t launch_twiddles(void *tw_f, void *tw_d, cudaStream_t st);
 // the plain FP32 table (same layout, the FP64 value rounded to float2)

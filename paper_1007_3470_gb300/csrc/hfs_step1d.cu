@@ -2,6 +2,8 @@
 // (FP32 and FP64, perturbation kind and box symmetry read per instance), the
 // launch dispatcher over the specialised FP32 variants, the norm / energy
 // diagnostics and the twiddle tables.
+#include <algorithm>
+
 #include "hfs_step1d.cuh"
 
 namespace hfs {
@@ -19,71 +21,180 @@ HFS_STEP1D_VARIANT(extern, float, HFS_VI_COS, true)
 // ---------------------------------------------------------------------------
 // diagnostics: norm and energy (FP64 accumulation)
 // ---------------------------------------------------------------------------
+// the sum over a team's threads (teams of T threads are aligned): in shuffles,
+// then the team's warps through slots
+template <int T> __device__ __forceinline__ double team_sum(double s, double *slots)
+{
+    constexpr int W = T < 32 ? T : 32;
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if constexpr (T > 32) {
+        const int bar = 1 + threadIdx.x / T, w0 = (threadIdx.x / T) * (T / 32);
+        exchange_sync<T, true>(bar);
+        if ((threadIdx.x & 31) == 0) slots[threadIdx.x >> 5] = s;
+        exchange_sync<T, true>(bar);
+        s = 0.0;
+#pragma unroll
+        for (int w = 0; w < T / 32; ++w) s += slots[w0 + w];
+    }
+    return s;
+}
+
+// Norm alone: one pass over the state, bound by the FP64 pipe (two FMAs and two
+// conversions a point at 2 lanes a cycle) a little above the memory time.
+template <typename R, int T, int E>
+__device__ __forceinline__ void norm_item(const Diag1DArgs &a, const WorkItem &it, double *slots)
+{
+    const int g = threadIdx.x / T, t = threadIdx.x - g * T;
+    const bool active = g < it.count;
+    const int idx = a.order[it.first + (active ? g : 0)];
+    const DevInst &ip = a.inst[idx];
+    const cpx<R> *psi = reinterpret_cast<const cpx<R> *>(a.psi) + ip.off;
+    double s = 0.0;
+    if (active) {
+        cpx<R> v[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = psi[t + T * e];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const double x = v[e].x, y = v[e].y;
+            s = fma(x, x, fma(y, y, s));
+        }
+    }
+    s = team_sum<T>(s, slots);
+    if (active && t == 0) a.out[2 * idx] = s * ip.dx[0];
+}
+
+// FP32 pairs hi + lo: sum += m2 |v|^2, every product and the sum exact to 2^-48
+struct Sum2 {
+    float hi = 0.0f, lo = 0.0f;
+};
+__device__ __forceinline__ void add_m2_abs2(Sum2 &s, float m2, cpx<float> v)
+{
+    const float p = v.x * v.x, q = v.y * v.y;
+    const float pq = p + q, bb = pq - p;
+    const float lo = (p - (pq - bb)) + (q - bb) + fmaf(v.x, v.x, -p) + fmaf(v.y, v.y, -q);
+    const float t = m2 * pq;
+    const float tl = fmaf(m2, lo, fmaf(m2, pq, -t));
+    const float h = s.hi + t, hb = h - s.hi;
+    s.lo += (s.hi - (h - hb)) + (t - hb) + tl;
+    s.hi = h;
+}
+
+// Energy.  Bound by the FP64 pipe: the potential's sum takes eight FP64
+// instructions a point (cos k x by c_{e+1} = 2 cos(k T dx) c_e - c_{e-1} over the
+// thread's points instead of cos; its error of some E^2 roundings is far below
+// the transform's), the kinetic sum of an FP32 state is formed in FP32 pairs.
+// 4096 mixed-size FP32 instances: norm and energy took 1.19 ms together (0.32 ms
+// now, copies included) as two runs of one kernel with cos and all sums in FP64.
 template <typename R, int N, int E, bool ALT>
-__device__ __forceinline__ void diag_item(const Diag1DArgs &a, const WorkItem &it, cpx<R> *smem)
+__device__ __forceinline__ void energy_item(const Diag1DArgs &a, const WorkItem &it, cpx<R> *smem, double *slots)
 {
     constexpr int T = N / E;
     const int g = threadIdx.x / T;
     const int t = threadIdx.x - g * T;
     const bool active = g < it.count;
+    if ((threadIdx.x & ~31) / T >= it.count) return;  // no instance in this warp
     const int idx = a.order[it.first + (active ? g : 0)];
     const DevInst &ip = a.inst[idx];
     const cpx<R> *psi = reinterpret_cast<const cpx<R> *>(a.psi) + ip.off;
     cpx<R> *sm = smem + g * smem_elems(N);
     const auto *tw = reinterpret_cast<const typename TwOf<R>::type *>(a.tw);
-    const double w2 = law_omega2(ip, *a.t_dev);
     cpx<R> v[E];
-    double nrm = 0.0, pot = 0.0, inter = 0.0, kin = 0.0;
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-        v[e] = active ? psi[t + T * e] : cpx<R>{R(0), R(0)};
-        const double x = ip.xc[0] + (double)(t + T * e - N / 2) * ip.dx[0];
-        const double d = (double)v[e].x * v[e].x + (double)v[e].y * v[e].y;
-        nrm += d;
-        pot += (0.5 * ip.mu * w2 * x * x + ip.eps * vi_eval(ip.vi_kind, x, ip.vi_k)) * d;
-        inter += 0.5 * ip.sigma * d * d;
-    }
-    FftPlan<N, E, ALT>::template run<false, R>(v, sm, t, tw);
-    const double kunit = 2.0 * 3.14159265358979323846 / ip.len[0];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int k = t + T * e;
-        const double kk = kunit * (double)((k < N / 2) ? k : k - N);
-        kin += kk * kk * ((double)v[e].x * v[e].x + (double)v[e].y * v[e].y);
-    }
-    const double energy = kin / N / (2.0 * ip.mu) + pot + inter;
-    __syncthreads();
-    double *red = reinterpret_cast<double *>(smem);
-    red[2 * threadIdx.x] = nrm;
-    red[2 * threadIdx.x + 1] = energy;
-    __syncthreads();
-    if (active && t == 0) {
-        double sn = 0.0, se = 0.0;
-        for (int u = 0; u < T; ++u) {
-            sn += red[2 * (threadIdx.x + u)];
-            se += red[2 * (threadIdx.x + u) + 1];
+    for (int e = 0; e < E; ++e) v[e] = active ? psi[t + T * e] : cpx<R>{R(0), R(0)};
+    double pot = 0.0;
+    if (active) {
+        const StageFGE pre = a.pre[idx];
+        const double c2 = pre.f, hs = 0.5 * ip.sigma, step = T * ip.dx[0];
+        const int kind = ip.eps != 0.0 ? ip.vi_kind : HFS_VI_NONE;
+        double x = ip.xc[0] + (double)(t - N / 2) * ip.dx[0];
+        double c = 0.0, cn = 0.0, f = 0.0;
+        if (kind == HFS_VI_COS) {
+            double sn, cs;
+            sincos(ip.vi_k * x, &sn, &cs);
+            f = 2.0 * pre.g;
+            c = ip.eps * cs;
+            cn = ip.eps * (cs * pre.g - sn * pre.e);
         }
-        a.out[2 * idx] = sn * ip.dx[0];
-        a.out[2 * idx + 1] = se * ip.dx[0];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const double vx = v[e].x, vy = v[e].y;
+            const double d = fma(vx, vx, vy * vy), xx = x * x;
+            double w = fma(hs, d, c2 * xx);
+            if (kind == HFS_VI_COS) {
+                w += c;
+                const double next = fma(f, cn, -c);
+                c = cn;
+                cn = next;
+            } else if (kind == HFS_VI_X4) {
+                w = fma(ip.eps * xx, xx, w);
+            }
+            pot = fma(w, d, pot);
+            x += step;
+        }
     }
-    __syncthreads();
+    FftPlan<N, E, ALT>::template run<false, R, 1, true>(v, sm, t, tw, 1 + g);
+    const double ku = 2.0 * 3.14159265358979323846 / ip.len[0], ck = ku * ku / N / (2.0 * ip.mu);
+    bool pairs = sizeof(R) == 4;
+    double s = 0.0;
+    if constexpr (sizeof(R) == 4) {
+        Sum2 kin;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const float m = (float)(t + T * e - (2 * e < E ? 0 : N));
+            add_m2_abs2(kin, m * m, v[e]);
+        }
+        s = team_sum<T>((double)kin.hi + (double)kin.lo, slots);
+        // pairs hold 48 bits while squares stay clear of FP32's range; a state of
+        // another size (or not finite) is summed in FP64
+        pairs = !active || (s > 1e-18 && s < 1e30);
+        if constexpr (T < 32) pairs = __all_sync(0xffffffffu, pairs);
+    }
+    if (!pairs) {
+        double kin = 0.0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int m = t + T * e - (2 * e < E ? 0 : N);
+            const double vx = v[e].x, vy = v[e].y;
+            kin = fma(square64(m), fma(vx, vx, vy * vy), kin);
+        }
+        s = team_sum<T>(kin, slots);
+    }
+    s = fma(s, ck, team_sum<T>(pot, slots));
+    if (active && t == 0) a.out[2 * idx + 1] = s * ip.dx[0];
 }
 
-template <typename R> __global__ void __launch_bounds__(kCtaThreads) diag1d_kernel(const Diag1DArgs a)
+// What every thread of an instance needs, once per instance: mu omega^2 / 2 and
+// cos, sin of k T dx (with the law's sine and this sincos in every thread the two
+// calls took 0.34 ms)
+__global__ void energy_pre_kernel(const Diag1DArgs a)
+{
+    const int w = blockIdx.x, i = threadIdx.x;
+    const WorkItem it = a.work[w];
+    if (i >= it.count) return;
+    const int idx = a.order[it.first + i];
+    const DevInst &ip = a.inst[idx];
+    StageFGE r{};
+    r.f = 0.5 * ip.mu * law_omega2(ip, *a.t_dev);
+    sincos(ip.vi_k * (ip.dx[0] * (ip.n[0] / plan_ept(it.plan))), &r.e, &r.g);
+    a.pre[idx] = r;
+}
+
+// items of a batch hold the same number of points each but for the last of a
+// grid size, so CTAs take them in turn
+template <typename R, bool ENERGY> __global__ void __launch_bounds__(kCtaThreads) diag1d_kernel(const Diag1DArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cpx<R> *smem = reinterpret_cast<cpx<R> *>(smem_raw);
-    __shared__ int s_item;
-    for (;;) {
-        if (threadIdx.x == 0) s_item = (int)atomicAdd(a.ticket, 1u);
-        __syncthreads();
-        const int w = s_item;
-        if (w >= a.nwork) break;
+    __shared__ double slots[kCtaThreads / 32];
+    for (int w = blockIdx.x; w < a.nwork; w += gridDim.x) {
         const WorkItem it = a.work[w];
         switch (it.plan) {
 #define HFS_CASE(NN, EE, AA)                                                                                      \
     case plan_id(NN, EE, AA):                                                                                     \
-        diag_item<R, NN, EE, AA>(a, it, smem);                                                                    \
+        if constexpr (ENERGY) energy_item<R, NN, EE, AA>(a, it, smem, slots);                                      \
+        else norm_item<R, NN / EE, EE>(a, it, slots);                                                             \
         break;
             HFS_FOR_EACH_PLAN(HFS_CASE)
             HFS_FOR_EACH_WIDE_PLAN(HFS_CASE)
@@ -141,16 +252,22 @@ size_t step1d_smem_bytes(bool fp64)
     return ((size_t)2 * step1d_exchange_elems + step1d_vtable_elems) * r + step1d_slot_floats * sizeof(float);
 }
 
-static cudaError_t prepare_diag(bool fp64)
+template <typename R, bool ENERGY> static cudaError_t diag_t(const Diag1DArgs &a, int sms, cudaStream_t st)
 {
-    static bool done[2] = {false, false};
-    if (done[fp64]) return cudaSuccess;
-    const int bytes = (int)step1d_smem_bytes(fp64);
-    const cudaError_t e =
-        fp64 ? cudaFuncSetAttribute(diag1d_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)
-             : cudaFuncSetAttribute(diag1d_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) done[fp64] = true;
-    return e;
+    // the exchange buffers of the step kernels without the table behind them
+    const int bytes = ENERGY ? (int)(step1d_exchange_elems * sizeof(cpx<R>)) : 0;
+    static int per_sm = 0;
+    if (!per_sm) {
+        cudaError_t e = cudaFuncSetAttribute(diag1d_kernel<R, ENERGY>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        int n = 0;
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, diag1d_kernel<R, ENERGY>, kCtaThreads, bytes);
+        if (e != cudaSuccess) return e;
+        per_sm = std::max(1, n);
+    }
+    if (ENERGY) energy_pre_kernel<<<a.nwork, 64, 0, st>>>(a);  // at most 64 instances an item
+    diag1d_kernel<R, ENERGY><<<std::max(1, std::min(a.nwork, sms * per_sm)), kCtaThreads, bytes, st>>>(a);
+    return cudaGetLastError();
 }
 
 template <bool WIDE> static int ctas_per_sm_f(int variant)
@@ -201,14 +318,10 @@ int step1d_variant(const hfs_instance *inst, int64_t count)
     return k;
 }
 
-cudaError_t launch_diag1d(bool fp64, const Diag1DArgs &a, int grid, cudaStream_t st)
+cudaError_t launch_diag1d(bool fp64, bool energy, const Diag1DArgs &a, int sms, cudaStream_t st)
 {
-    cudaError_t e = prepare_diag(fp64);
-    if (e != cudaSuccess) return e;
-    const size_t bytes = step1d_smem_bytes(fp64);
-    if (fp64) diag1d_kernel<double><<<grid, kCtaThreads, bytes, st>>>(a);
-    else diag1d_kernel<float><<<grid, kCtaThreads, bytes, st>>>(a);
-    return cudaGetLastError();
+    if (fp64) return energy ? diag_t<double, true>(a, sms, st) : diag_t<double, false>(a, sms, st);
+    return energy ? diag_t<float, true>(a, sms, st) : diag_t<float, false>(a, sms, st);
 }
 
 cudaError_t launch_twiddles_plain(void *tw_p, cudaStream_t st)

@@ -53,3 +53,37 @@ def test_fp64_phases(vi, shift, split):
     need_gpu()
     insts, psis = _instances(512, 2, vi, shift, seed=7)
     assert _worst(insts, psis, 6, "c128", split=split, h=0.02, scheme="ni4_82") <= budget(TOL_C128, 0.12)
+
+
+@pytest.mark.parametrize("precision", ["c64", "c128"])
+@pytest.mark.parametrize("scale", [1.0, 1e-17, 1e17])
+@pytest.mark.parametrize("vi,shift", [(W.VI_COS, False), (W.VI_COS, True), (W.VI_X4, True), (W.VI_NONE, False)])
+def test_norm_and_energy(precision, scale, vi, shift):
+    """Norm and energy of a mixed batch against numpy in FP64, for states whose
+    squares leave FP32's range as well.  The norm is an FP64 sum of the stored
+    values (n roundings, 1e-12 allowed); the energy of an FP32 state carries the
+    transform's FP32 roundings (1e-6), of an FP64 state none (1e-12)."""
+    need_gpu()
+    from paper_1007_3470_gb300 import hfs
+    insts, psis = [], []
+    for n in (128, 256, 512, 1024, 2048, 4096):
+        i, p = _instances(n, 3, vi, shift, seed=n)
+        insts += i
+        psis += p
+    psis = [np.asarray(p * scale).astype(np.complex64 if precision == "c64" else np.complex128) for p in psis]
+    s = hfs.Solver(insts, precision=precision, chunk_steps=4)
+    s.set_psi(psis)
+    norm, energy = s.norm(), s.energy()
+    s.close()
+    for i, inst in enumerate(insts):
+        u = psis[i].astype(np.complex128)
+        x, n = inst.x(), inst.n[0]
+        dx = x[1] - x[0]
+        d = np.abs(u) ** 2
+        v = {W.VI_NONE: 0 * x, W.VI_X4: x ** 4, W.VI_COS: np.cos(inst.vi_k * x)}[vi]
+        k = 2 * np.pi * np.fft.fftfreq(n, dx)
+        kin = 0.5 * np.sum(np.abs(k * np.fft.fft(u)) ** 2) / n
+        w0 = inst.w0 * (1 + inst.law[0] * np.sin(inst.law[2]))
+        want = dx * (kin + np.sum((0.5 * w0 ** 2 * x ** 2 + inst.eps * v) * d + 0.5 * inst.sigma * d * d))
+        assert abs(norm[i] - dx * d.sum()) <= 1e-12 * dx * d.sum()
+        assert abs(energy[i] - want) <= (1e-6 if precision == "c64" else 1e-12) * abs(want), (n, i)
