@@ -197,20 +197,49 @@ __global__ void law_nodes_kernel(const DevInst *__restrict__ inst, SchedConst sc
     nodes[sg] = stage_nodes<FLOW, LAW>(inst[0], tau, sc.a[st] * sc.h);
 }
 
+// Work of a thread of the schedule kernels: (instance, entry of its chunk).  A
+// block takes one instance (x) and strides over its entries (y), or, where a
+// chunk has fewer than kFlatBelow entries an instance, threads take instances
+// and entries in one line (with an integer division each; one block of 128 for
+// every instance left 127 threads idle on calls of one step: 65 + 45 us for
+// 16384 instances).
+constexpr int kFlatBelow = 64;
+struct ItemAt {
+    int64_t i;
+    int n, stride;  // stride 0: none of this thread's
+};
+template <bool FLAT> __device__ __forceinline__ ItemAt item_at(int64_t count, int per)
+{
+    if constexpr (FLAT) {
+        const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+        if (u >= count * per) return {0, 0, 0};
+        const int64_t i = u < ((int64_t)1 << 32) ? (int64_t)((unsigned)u / (unsigned)per) : u / per;
+        return {i, (int)(u - i * per), per};
+    } else {
+        return {(int64_t)blockIdx.x, (int)(blockIdx.y * blockDim.x + threadIdx.x), (int)(gridDim.y * blockDim.x)};
+    }
+}
+static dim3 item_grid(int64_t count, int64_t per, bool flat)
+{
+    if (flat) return dim3((unsigned)((count * per + 127) / 128));
+    return dim3((unsigned)count, (unsigned)std::min<int64_t>((per + 127) / 128, 65535));
+}
+
 // one thread per (instance, time step of the chunk), all m stages of the
-// step: instance = blockIdx.x, steps strided over blockIdx.y / threadIdx.x
-// (no 64-bit integer division in the index arithmetic).  SHARED: the shape
-// factors come from law_nodes_kernel instead of being evaluated per instance.
-template <int FLOW, int LAW, bool SHARED>
-__global__ void stage_flow_kernel(const DevInst *__restrict__ inst, int dim, SchedConst sc,
+// step.  SHARED: the shape factors come from law_nodes_kernel instead of being
+// evaluated per instance.
+template <int FLOW, int LAW, bool SHARED, bool FLAT>
+__global__ void stage_flow_kernel(const DevInst *__restrict__ inst, int64_t count, int dim, SchedConst sc,
                                   const double *__restrict__ t_dev, double t_off, int nsteps,
                                   const NodeS *__restrict__ nodes, StageFGE *__restrict__ out, unsigned *status)
 {
-    const int64_t i = blockIdx.x;
-    const DevInst p = inst[i];
+    const ItemAt at = item_at<FLAT>(count, nsteps);
+    if (FLAT && at.stride == 0) return;
+    const int64_t i = at.i;
+    const DevInst &p = inst[i];
     const double t0 = *t_dev + t_off;
     const int64_t nstage = (int64_t)nsteps * sc.m;
-    for (int n = blockIdx.y * blockDim.x + threadIdx.x; n < nsteps; n += gridDim.y * blockDim.x) {
+    for (int n = at.n; n < nsteps; n += at.stride) {
         for (int st = 0; st < sc.m; ++st) {
             const double tau = t0 + (double)n * sc.h + sc.h * sc.cuma[st];
             const double s = sc.a[st] * sc.h;
@@ -291,16 +320,23 @@ __device__ __forceinline__ void record1d(const DevInst &p, const SchedConst &sc,
     double kappa, bs, g;
     merged_coeffs<SPLIT>(p, 1, 0, sc, t0, j, nstage, fge_i, kappa, bs, g);
     const double K2 = kappa * c.k2;
-    const double K1 = kappa * c.k1;
-    const double K0 = frac1(kappa * c.k0);
     const double G = g * c.g;
     const double SB = bs * c.sb;
+    // the terms of an off-centre box (half of a record's FP64 work)
+    double K1 = 0.0, K0 = 0.0;
+    if (c.k1 != 0.0) {
+        K1 = kappa * c.k1;
+        K0 = frac1(kappa * c.k0);
+    }
     if (!isfinite(K2) || !isfinite(G) || !isfinite(K1)) atomicOr(status, (unsigned)ST_NONFINITE);
     RecT r;
     if constexpr (sizeof(RecT) == sizeof(RecF)) {
         split_hi_lo(K2, r.k2hi, r.k2lo);
-        split_hi_lo(K1, r.k1hi, r.k1lo);
-        r.k0 = (float)K0;
+        r.k1hi = r.k1lo = r.k0 = 0.0f;
+        if (c.k1 != 0.0) {
+            split_hi_lo(K1, r.k1hi, r.k1lo);
+            r.k0 = (float)K0;
+        }
         r.sb2pi = (float)SB;
         split_hi_lo(G, r.ghi, r.glo);
     } else {
@@ -314,23 +350,29 @@ __device__ __forceinline__ void record1d(const DevInst &p, const SchedConst &sc,
     *out = r;
 }
 
-// one thread per (instance, sub-stage j in [0, nstage]) -- 1D records;
-// instance = blockIdx.x, sub-stages strided over blockIdx.y / threadIdx.x
-template <typename RecT, int SPLIT>
-__global__ void records1d_kernel(const DevInst *__restrict__ inst, SchedConst sc, const double *__restrict__ t_dev,
-                                 double t_off, int nstage, const StageFGE *__restrict__ fge, RecT *__restrict__ rec,
-                                 unsigned *status)
+// one thread per (instance, sub-stage j in [0, nstage]) -- 1D records
+template <typename RecT, int SPLIT, bool FLAT>
+__global__ void records1d_kernel(const DevInst *__restrict__ inst, int64_t count, SchedConst sc,
+                                 const double *__restrict__ t_dev, double t_off, int nstage,
+                                 const StageFGE *__restrict__ fge, RecT *__restrict__ rec, unsigned *status)
 {
-    const int64_t i = blockIdx.x;
     const int64_t nrec = (int64_t)nstage + 1;
-    const DevInst p = inst[i];
+    const ItemAt at = item_at<FLAT>(count, (int)nrec);
+    if (FLAT && at.stride == 0) return;
+    const int64_t i = at.i;
+    const DevInst &p = inst[i];
     const double t0 = *t_dev + t_off;
-    // the block's instance factors, computed once (one FP64 division per block, not per record)
-    __shared__ RecScale s_c;
-    if (threadIdx.x == 0) s_c = rec_scale(p, sc);
-    __syncthreads();
-    const RecScale c = s_c;
-    for (int j = blockIdx.y * blockDim.x + threadIdx.x; j <= nstage; j += gridDim.y * blockDim.x)
+    RecScale c;
+    if constexpr (FLAT) {
+        c = rec_scale(p, sc);
+    } else {
+        // the block's instance factors, computed once (one FP64 division per block, not per record)
+        __shared__ RecScale s_c;
+        if (threadIdx.x == 0) s_c = rec_scale(p, sc);
+        __syncthreads();
+        c = s_c;
+    }
+    for (int j = at.n; j <= nstage; j += at.stride)
         record1d<RecT, SPLIT>(p, sc, c, t0, j, nstage, fge + i * (int64_t)nstage, rec + i * nrec + j, status);
 }
 
@@ -395,30 +437,40 @@ bool law_shared(const hfs_instance *inst, int64_t count)
 size_t law_nodes_bytes(int64_t nstage) { return sizeof(NodeS) * (size_t)nstage; }
 
 template <int FLOW, int LAW>
-static void launch_stage_flow_fl(bool shared, dim3 grid, const DevInst *inst, int dim, const SchedConst &sc,
+static void launch_stage_flow_fl(bool shared, const DevInst *inst, int64_t count, int dim, const SchedConst &sc,
                                  const double *t_dev, double t_off, int nsteps, void *nodes, StageFGE *out,
                                  unsigned *status, cudaStream_t st)
 {
     NodeS *nd = static_cast<NodeS *>(nodes);
+    const bool flat = nsteps < kFlatBelow;
+    const dim3 grid = item_grid(count, nsteps, flat);
     if constexpr (LAW >= 0) {
         if (shared && nd) {
             const int nstage = nsteps * sc.m;
             law_nodes_kernel<FLOW, LAW><<<blocks_for(nstage, 128), 128, 0, st>>>(inst, sc, t_dev, t_off, nstage, nd);
-            stage_flow_kernel<FLOW, LAW, true><<<grid, 128, 0, st>>>(inst, dim, sc, t_dev, t_off, nsteps, nd, out,
-                                                                      status);
+            if (flat)
+                stage_flow_kernel<FLOW, LAW, true, true>
+                    <<<grid, 128, 0, st>>>(inst, count, dim, sc, t_dev, t_off, nsteps, nd, out, status);
+            else
+                stage_flow_kernel<FLOW, LAW, true, false>
+                    <<<grid, 128, 0, st>>>(inst, count, dim, sc, t_dev, t_off, nsteps, nd, out, status);
             return;
         }
     }
-    stage_flow_kernel<FLOW, LAW, false><<<grid, 128, 0, st>>>(inst, dim, sc, t_dev, t_off, nsteps, nullptr, out,
-                                                               status);
+    if (flat)
+        stage_flow_kernel<FLOW, LAW, false, true>
+            <<<grid, 128, 0, st>>>(inst, count, dim, sc, t_dev, t_off, nsteps, nullptr, out, status);
+    else
+        stage_flow_kernel<FLOW, LAW, false, false>
+            <<<grid, 128, 0, st>>>(inst, count, dim, sc, t_dev, t_off, nsteps, nullptr, out, status);
 }
 
 template <int FLOW>
-static void launch_stage_flow_law(int law, bool shared, dim3 grid, const DevInst *inst, int dim, const SchedConst &sc,
-                                  const double *t_dev, double t_off, int nsteps, void *nodes, StageFGE *out,
-                                  unsigned *status, cudaStream_t st)
+static void launch_stage_flow_law(int law, bool shared, const DevInst *inst, int64_t count, int dim,
+                                  const SchedConst &sc, const double *t_dev, double t_off, int nsteps, void *nodes,
+                                  StageFGE *out, unsigned *status, cudaStream_t st)
 {
-#define HFS_SF(L) launch_stage_flow_fl<FLOW, L>(shared, grid, inst, dim, sc, t_dev, t_off, nsteps, nodes, out, status, st)
+#define HFS_SF(L) launch_stage_flow_fl<FLOW, L>(shared, inst, count, dim, sc, t_dev, t_off, nsteps, nodes, out, status, st)
     switch (law) {
     case HFS_OMEGA_CONST: HFS_SF(HFS_OMEGA_CONST); break;
     case HFS_OMEGA_SIN: HFS_SF(HFS_OMEGA_SIN); break;
@@ -436,19 +488,18 @@ cudaError_t launch_stage_flow(const DevInst *inst, int64_t count, int dim, const
     if (count == 0 || nstage == 0) return cudaSuccess;
     if (nstage >= INT32_MAX || nstage % sc.m != 0 || count > INT32_MAX) return cudaErrorInvalidValue;
     const int nsteps = (int)(nstage / sc.m);
-    const dim3 grid((unsigned)count, std::min(blocks_for(nsteps, 128), 65535u));
     switch (sc.flow) {
     case HFS_FLOW_LEMMA2:
-        launch_stage_flow_law<HFS_FLOW_LEMMA2>(uniform_law, shared, grid, inst, dim, sc, t_dev, t_off, nsteps, nodes,
-                                               out, status, st);
+        launch_stage_flow_law<HFS_FLOW_LEMMA2>(uniform_law, shared, inst, count, dim, sc, t_dev, t_off, nsteps,
+                                               nodes, out, status, st);
         break;
     case HFS_FLOW_CF4:
-        launch_stage_flow_law<HFS_FLOW_CF4>(uniform_law, shared, grid, inst, dim, sc, t_dev, t_off, nsteps, nodes,
-                                            out, status, st);
+        launch_stage_flow_law<HFS_FLOW_CF4>(uniform_law, shared, inst, count, dim, sc, t_dev, t_off, nsteps,
+                                               nodes, out, status, st);
         break;
     default:
-        launch_stage_flow_law<HFS_FLOW_M6>(uniform_law, shared, grid, inst, dim, sc, t_dev, t_off, nsteps, nodes,
-                                           out, status, st);
+        launch_stage_flow_law<HFS_FLOW_M6>(uniform_law, shared, inst, count, dim, sc, t_dev, t_off, nsteps,
+                                               nodes, out, status, st);
         break;
     }
     return cudaGetLastError();
@@ -460,16 +511,20 @@ cudaError_t launch_records1d(bool fp64, const DevInst *inst, int64_t count, cons
 {
     if (count == 0) return cudaSuccess;
     if (nstage >= INT32_MAX || count > INT32_MAX) return cudaErrorInvalidValue;
-    const dim3 grid((unsigned)count, std::min(blocks_for(nstage + 1, 128), 65535u));
-    const bool ho = sc.split == HFS_SPLIT_HO;
-    if (fp64 && ho)
-        records1d_kernel<RecD, HFS_SPLIT_HO><<<grid, 128, 0, st>>>(inst, sc, t_dev, t_off, (int)nstage, fge, (RecD *)rec, status);
-    else if (fp64)
-        records1d_kernel<RecD, HFS_SPLIT_FOURIER><<<grid, 128, 0, st>>>(inst, sc, t_dev, t_off, (int)nstage, fge, (RecD *)rec, status);
-    else if (ho)
-        records1d_kernel<RecF, HFS_SPLIT_HO><<<grid, 128, 0, st>>>(inst, sc, t_dev, t_off, (int)nstage, fge, (RecF *)rec, status);
-    else
-        records1d_kernel<RecF, HFS_SPLIT_FOURIER><<<grid, 128, 0, st>>>(inst, sc, t_dev, t_off, (int)nstage, fge, (RecF *)rec, status);
+    const bool ho = sc.split == HFS_SPLIT_HO, flat = nstage + 1 < kFlatBelow;
+    const dim3 grid = item_grid(count, nstage + 1, flat);
+    auto launch = [&](auto kernel, auto *r) {
+        kernel<<<grid, 128, 0, st>>>(inst, count, sc, t_dev, t_off, (int)nstage, fge, r, status);
+    };
+    if (fp64) {
+        RecD *r = (RecD *)rec;
+        if (ho) flat ? launch(records1d_kernel<RecD, HFS_SPLIT_HO, true>, r) : launch(records1d_kernel<RecD, HFS_SPLIT_HO, false>, r);
+        else flat ? launch(records1d_kernel<RecD, HFS_SPLIT_FOURIER, true>, r) : launch(records1d_kernel<RecD, HFS_SPLIT_FOURIER, false>, r);
+    } else {
+        RecF *r = (RecF *)rec;
+        if (ho) flat ? launch(records1d_kernel<RecF, HFS_SPLIT_HO, true>, r) : launch(records1d_kernel<RecF, HFS_SPLIT_HO, false>, r);
+        else flat ? launch(records1d_kernel<RecF, HFS_SPLIT_FOURIER, true>, r) : launch(records1d_kernel<RecF, HFS_SPLIT_FOURIER, false>, r);
+    }
     return cudaGetLastError();
 }
 
