@@ -72,6 +72,23 @@ int composition_fixed(int comp, double *a, double *b, int *m)
     }
 }
 
+// Values per thread where no plan was set (batches that small1d_ok leaves).  16
+// for large batches of one size, but for 512 points (three radix-8 passes: 11.5
+// against 12.6 us a step of 4096 instances).  8, on twice the threads, while these
+// make at most two 256-thread CTAs an SM (608 instances of 1024 points 4.05
+// against 4.78 us a step, 1216 of them 7.7 against 6.7), and for the sizes up to
+// 1024 of a mixed batch: their shorter, more numerous warps fill the gaps that
+// the long transforms' exchanges leave (4096 instances of 128 ... 4096 points, 200
+// steps: 7.64 -> 7.05 ms, 6.21 -> 5.93 ms with the norm projection).  FP64: 8 until
+// the FP64 pipe has eight warps an SM (one instance of 1024 points: 63 -> 35 us a
+// sub-stage).
+int default_ept(int n, int64_t points, bool mixed, int sms, bool fp64)
+{
+    if (n <= 2048 && points / 8 <= (int64_t)sms * kCtaThreads * (fp64 ? 1 : 2)) return 8;
+    if (!fp64 && n <= 1024 && (mixed || n == 512)) return 8;
+    return 16;
+}
+
 // upper bound of omega over [t0, t1] for the validity check
 double omega_bound(const hfs_instance &p, double t0, double t1)
 {
@@ -113,6 +130,7 @@ struct hfs_ctx_s {
     // alternative radix order (16 only); CTAs per SM of the step grid (0: as
     // many as fit)
     int ept[kNumSizes] = {16, 16, 16, 16, 16, 16};
+    bool plan_set[kNumSizes] = {};  // by the caller or the autotuner; the others follow default_ept
     bool alt[kNumSizes] = {false, false, false, false, false, false};
     int ctas_per_sm = 0;
     // trap law shared by every instance (HFS_OMEGA_*), -1 for a mixed batch,
@@ -121,6 +139,7 @@ struct hfs_ctx_s {
     bool law_shared = false;
     // specialised 1D step kernel (step1d_variant), -1 for the generic one
     int variant = -1;
+    bool small = false;  // few complex64 instances without set plans (small1d_ok)
     std::vector<int32_t> order;  // sorted position -> instance
     std::vector<WorkItem> work;
     // schedule
@@ -199,7 +218,7 @@ Layout make_layout(const hfs_ctx_s *c, int64_t chunk)
     const size_t recsz = (c->dim == 1) ? (c->precision == HFS_C128 ? sizeof(RecD) : sizeof(RecF))
                                        : (c->precision == HFS_C128 ? sizeof(Rec3D) : sizeof(Rec3F));
     L.status = take(sizeof(unsigned));
-    L.ticket = take(sizeof(unsigned));
+    L.ticket = take(2 * sizeof(unsigned));  // work ticket, counter of launch_small1d
     L.tdev = take(sizeof(double));
     L.inst = take(sizeof(DevInst) * c->count);
     L.order = take(sizeof(int32_t) * c->count);
@@ -229,11 +248,14 @@ void build_worklist(hfs_ctx_s *c)
     std::stable_sort(c->order.begin(), c->order.end(),
                      [&](int32_t x, int32_t y) { return c->inst[x].n[0] > c->inst[y].n[0]; });
     c->work.clear();
+    c->small = c->precision == HFS_C64 && small1d_ok(c->dinst.data(), c->count, c->elems, c->sm_count);
+    for (auto &p : c->inst) c->small = c->small && !c->plan_set[size_class(p.n[0])];
+    const bool fp64 = c->precision == HFS_C128, mixed = c->inst[c->order[0]].n[0] != c->inst[c->order[c->count - 1]].n[0];
     int64_t i = 0;
     while (i < c->count) {
         const int n = c->inst[c->order[i]].n[0];
-        const int e = c->ept[size_class(n)];
-        const bool alt = c->alt[size_class(n)];
+        const bool set = c->plan_set[size_class(n)], alt = set && c->alt[size_class(n)];
+        const int e = set ? c->ept[size_class(n)] : default_ept(n, c->elems, mixed, c->sm_count, fp64);
         const int per = kCtaThreads / (n / e);
         int64_t j = i;
         while (j < c->count && j - i < per && c->inst[c->order[j]].n[0] == n) ++j;
@@ -241,7 +263,7 @@ void build_worklist(hfs_ctx_s *c)
         w.first = (int32_t)i;
         w.count = (int32_t)(j - i);
         w.plan = plan_id(n, e, alt);
-        w.pad = 0;
+        w.diag = plan_id(n, set ? e : 16, alt);
         c->work.push_back(w);
         i = j;
     }
@@ -383,7 +405,10 @@ int enqueue_steps(hfs_ctx_s *c, int64_t nsteps, const ReusePlan &rp = ReusePlan(
         };
         // under schedule reuse a call is one chunk (done = 0, S = nsteps)
         void *rec_now = (rp.on && rp.cur == 1) ? wptr<void>(c, c->lay.rec2) : rec;
-        if (!rp.on || rp.compute) {
+        // one launch that makes its own records and advances the time
+        const bool own = c->small && !rp.on && S == nsteps && nstage <= kSmallSchedStages &&
+                         (c->mode == HFS_MODE_RESIDENT || c->spl >= S);
+        if (!own && (!rp.on || rp.compute)) {
             const int s = schedule(c->stream, toff, rec_now);
             if (s) return s;
         }
@@ -422,6 +447,11 @@ int enqueue_steps(hfs_ctx_s *c, int64_t nsteps, const ReusePlan &rp = ReusePlan(
                 a.final_x = (s1 == S) ? 1 : 0;
                 // the first launch of the call records the norm it projects onto
                 a.proj = !c->norm_projection ? PROJ_OFF : (done == 0 && s0 == 0) ? PROJ_SET : PROJ_USE;
+                if (c->small) {
+                    const Small1DArgs sa{a, (int32_t)c->count, own ? (int32_t)S : 0, c->sc, tdev, ticket + 1};
+                    CK(launch_small1d(sa, c->inst[c->order[0]].n[0], c->variant, c->stream, rp.prefetch ? c->prio_high : 0));
+                    continue;
+                }
                 CK(cudaMemsetAsync(ticket, 0, sizeof(unsigned), c->stream));
                 CK(launch_step1d(fp64, c->variant, a, grid, c->stream, wide, rp.prefetch ? c->prio_high : 0));
             }
@@ -448,6 +478,7 @@ int enqueue_steps(hfs_ctx_s *c, int64_t nsteps, const ReusePlan &rp = ReusePlan(
             if (c->profiling && done + S >= nsteps) CK(record_prof(c, 1));
         }
         done += S;
+        if (own) return HFS_OK;
     }
     CK(launch_advance_time(tdev, (double)nsteps * c->sc.h, c->stream));
     return HFS_OK;
@@ -554,13 +585,13 @@ int hfs_create(hfs_ctx_t *out, int dim, int precision, const hfs_instance *inst,
         if (dim == 1) set_1d_fp32_params(d);
     }
     c->elems = off;
-    if (dim == 1) build_worklist(c);
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         delete c;
         return HFS_ERR_CUDA;
     }
+    if (dim == 1) build_worklist(c);
     c->diag_host.resize(2 * count);
     *out = c;
     return HFS_OK;
@@ -644,6 +675,7 @@ int hfs_bind(hfs_ctx_t c, void *psi, void *work, size_t work_bytes, int64_t chun
     c->lay = L;
     (void)cudaGetLastError();
     CK(cudaMemsetAsync(wptr<void>(c, L.status), 0, sizeof(unsigned), c->stream));
+    CK(cudaMemsetAsync(wptr<void>(c, L.ticket), 0, 2 * sizeof(unsigned), c->stream));
     CK(cudaMemcpyAsync(wptr<void>(c, L.inst), c->dinst.data(), sizeof(DevInst) * c->count, cudaMemcpyHostToDevice,
                        c->stream));
     if (c->dim == 1) {
@@ -938,6 +970,7 @@ int hfs_set_plan(hfs_ctx_t c, int n, int plan)
     if ((ept == 4 || alt) && c->precision != HFS_C64) return HFS_ERR_UNSUPPORTED;
     c->ept[sc] = ept;
     c->alt[sc] = alt;
+    c->plan_set[sc] = true;
     build_worklist(c);
     drop_graphs(c);
     if (c->work_base) return upload_tables(c);
@@ -1004,6 +1037,7 @@ int autotune(hfs_ctx_s *c, int trial_steps, float *best_total)
     for (int k = 0; k < kNumSizes; ++k) {
         c->ept[k] = (128 << k) <= 1024 ? 8 : 16;
         c->alt[k] = false;
+        c->plan_set[k] = true;
     }
     build_worklist(c);
     s = time_worklist(c, steps, e0, e1, &total);

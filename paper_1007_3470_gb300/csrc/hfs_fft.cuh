@@ -253,9 +253,10 @@ template <int ILV> __host__ __device__ constexpr int soff(int c)
 // TEAM = true: only the T threads of the team that owns the buffer (named
 // barrier `bar`, or the warp when a team fits in one), so the teams of a CTA
 // holding several short transforms do not wait for one another.
-template <int T, bool TEAM> __device__ __forceinline__ void exchange_sync(int bar)
+// NAMED: a team that may be part of a larger CTA than kCtaThreads.
+template <int T, bool TEAM, bool NAMED = false> __device__ __forceinline__ void exchange_sync(int bar)
 {
-    if constexpr (!TEAM || T >= kCtaThreads) {
+    if constexpr (!TEAM || (T >= kCtaThreads && !NAMED)) {
         __syncthreads();
     } else if constexpr (T <= 32) {
         __syncwarp();
@@ -321,6 +322,145 @@ __device__ __forceinline__ void fft_passes(cpx<R> (&v)[E], cpx<R> *sm, int t,
     stockham_pass<N, E, RAD, NS, INV, sizeof...(REST) == 0, ILV, TEAM, R, TWC>(v, sm, t, tw, bar);
     if constexpr (sizeof...(REST) > 0)
         fft_passes<N, E, INV, ILV, TEAM, R, TWC, NS * RAD, REST...>(v, sm, t, tw, bar);
+}
+
+// ---------------------------------------------------------------------------
+// The transform of the plans with sixteen values per thread, on four threads
+// for each of theirs: every thread u = 4 b + q holds four values, positions
+// t + (N/4) e with t = b + (N/16) q, and a radix-16 butterfly b lies on four
+// adjacent lanes.  Its inner radix-4 transforms are local (lane q holds the
+// inputs q + 4 e), the twiddles W_16^{q k} depend on the lane, a 4 x 4 transpose
+// by shuffles feeds the outer ones.  A closing radix 8 lies on lanes q and q ^ 2,
+// radices 4 and 2 on one lane.  The operations on every value are those of
+// stockham_pass, in the same order, so the results are the same bits.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ cpx<float> shfl_xor(cpx<float> a, int m)
+{
+    return {__shfl_xor_sync(0xffffffffu, a.x, m), __shfl_xor_sync(0xffffffffu, a.y, m)};
+}
+// v[j] of lane k <-> v[k] of lane j, for four adjacent lanes
+__device__ __forceinline__ void lane_transpose4(cpx<float> (&v)[4], int q)
+{
+#pragma unroll
+    for (int m = 1; m <= 2; m <<= 1) {
+        const bool hi = q & m;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (i & m) continue;
+            const cpx<float> r = shfl_xor(hi ? v[i] : v[i | m], m);
+            if (hi) v[i] = r;
+            else v[i | m] = r;
+        }
+    }
+}
+// a W_16^{q K} on lane q: the forms of rot16 side by side and a selection (the
+// lanes' different branches one after the other took twice as long)
+template <int K, bool INV> __device__ __forceinline__ cpx<float> lane_rot16(cpx<float> a, int q)
+{
+    static_assert(K >= 1 && K <= 3, "inner transform's outputs");
+    if constexpr (K == 2) {
+        // exponents 0, 2, 4, 6
+        const cpx<float> w2 = rot16<2, INV>(a), w6 = rot16<6, INV>(a), w4 = rot16<4, INV>(a);
+        const cpx<float> lo = (q & 1) ? w2 : a, hi = (q & 1) ? w6 : w4;
+        return (q & 2) ? hi : lo;
+    } else {
+        // exponents 0, 1, 2, 3 (K = 1) and 0, 3, 6, 9: compensated products on the odd lanes
+        constexpr float C1H = 0.9238795042037964f, C1L = 2.830748968563057e-08f;
+        constexpr float S1H = 0.3826834261417389f, S1L = 6.2233507236442165e-09f;
+        const bool three = q & 2;
+        // lane 1: exponent K, lane 3: exponent 3 K
+        float ch, cl, sh, sl;
+        if constexpr (K == 1) {
+            ch = three ? S1H : C1H;
+            cl = three ? S1L : C1L;
+            sh = three ? -C1H : -S1H;
+            sl = three ? -C1L : -S1L;
+        } else {
+            ch = three ? -C1H : S1H;
+            cl = three ? -C1L : S1L;
+            sh = three ? S1H : -C1H;
+            sl = three ? S1L : -C1L;
+        }
+        if constexpr (INV) {
+            sh = -sh;
+            sl = -sl;
+        }
+        const cpx<float> m = mulw2(a, ch, cl, sh, sl), r = rot16<2 * K, INV>(a);
+        const cpx<float> even = (q & 2) ? r : a;
+        return (q & 1) ? m : even;
+    }
+}
+template <bool INV> __device__ __forceinline__ void lane_dft16(cpx<float> (&v)[4], int q)
+{
+    dft4s<INV, HFS_PACK_DFT16 != 0>(v[0], v[1], v[2], v[3]);
+    v[1] = lane_rot16<1, INV>(v[1], q);
+    v[2] = lane_rot16<2, INV>(v[2], q);
+    v[3] = lane_rot16<3, INV>(v[3], q);
+    lane_transpose4(v, q);
+    dft4s<INV, HFS_PACK_DFT16 != 0>(v[0], v[1], v[2], v[3]);
+}
+// radix 8 on lanes q (q & 2 == 0: even inputs) and q ^ 2 (odd inputs)
+template <bool INV> __device__ __forceinline__ void lane_dft8(cpx<float> (&v)[4], int q)
+{
+    const bool odd = q & 2;
+    dft4s<INV, HFS_PACK_DFT8 != 0>(v[0], v[1], v[2], v[3]);
+    if (odd) {
+        v[1] = rot16<2, INV>(v[1]);
+        v[2] = rot16<4, INV>(v[2]);
+        v[3] = rot16<6, INV>(v[3]);
+    }
+    __syncwarp();
+    // the even lane forms outputs 0, 2, 4, 6, the odd one 1, 3, 5, 7
+    const cpx<float> r0 = shfl_xor(odd ? v[0] : v[1], 2), r1 = shfl_xor(odd ? v[2] : v[3], 2);
+    const cpx<float> e0 = odd ? r0 : v[0], e1 = odd ? r1 : v[2], o0 = odd ? v[1] : r0, o1 = odd ? v[3] : r1;
+    v[0] = cadd(e0, o0);
+    v[1] = cadd(e1, o1);
+    v[2] = csub(e0, o0);
+    v[3] = csub(e1, o1);
+}
+
+template <int N, int RAD, int NS, bool INV, bool LAST>
+__device__ __forceinline__ void lane_pass(cpx<float> (&v)[4], cpx<float> *sm, int b, int q, const float4 *__restrict__ tw)
+{
+    constexpr int T = N / 4, T16 = N / 16;
+    const int t = b + T16 * q;
+    if constexpr (NS > 1) {
+        // position t + T e is input r of butterfly c: position = c + r N/RAD
+        constexpr int64_t OFF = tw_pass_offset(NS * RAD, RAD);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int pos = t + T * e, c = pos & (N / RAD - 1), r = pos / (N / RAD), j = c & (NS - 1);
+            if (r > 0) v[e] = tw_mul<INV>(v[e], tw, (int)OFF + (r - 1) * NS + j);
+        }
+        __syncwarp();
+    }
+    if constexpr (RAD == 16) lane_dft16<INV>(v, q);
+    else if constexpr (RAD == 8) lane_dft8<INV>(v, q);
+    else if constexpr (RAD == 4) dft4<INV>(v[0], v[1], v[2], v[3]);
+    else {
+        dft2<INV>(v[0], v[2]);
+        dft2<INV>(v[1], v[3]);
+    }
+    if constexpr (!LAST) {
+        static_assert(RAD == 16, "only radix-16 passes come before another");
+        const int j = b & (NS - 1);
+        cpx<float> *w = sm + sbase<1>((b - j) * 16 + j + q * NS);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[soff<1>(4 * k * NS)] = v[k];
+        exchange_sync<T, true, true>(1);
+        const cpx<float> *rd = sm + sbase<1>(t);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = rd[soff<1>(T * e)];
+        exchange_sync<T, true, true>(1);
+    }
+}
+template <int N, bool INV> __device__ __forceinline__ void lane_fft(cpx<float> (&v)[4], cpx<float> *sm, int b, int q, const float4 *tw)
+{
+    lane_pass<N, 16, 1, INV, false>(v, sm, b, q, tw);
+    if constexpr (N == 128) lane_pass<N, 8, 16, INV, true>(v, sm, b, q, tw);
+    else lane_pass<N, 16, 16, INV, N == 256>(v, sm, b, q, tw);
+    if constexpr (N > 256) lane_pass<N, N / 256, 256, INV, true>(v, sm, b, q, tw);
+    static_assert(N <= 1024, "radix sequence");
 }
 
 // Radix sequences per (N, elements per thread, ALT: the alternative order).

@@ -137,7 +137,7 @@ struct WorkItem {
     int32_t first;  // index into the sorted instance order
     int32_t count;  // instances in this item (<= instances per CTA)
     int32_t plan;   // plan id (grid size class + elements per thread)
-    int32_t pad;
+    int32_t diag;   // plan id of the diagnostics (16 values per thread unless a plan was set)
 };
 
 // supported 1D sizes

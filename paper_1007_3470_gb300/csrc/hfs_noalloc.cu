@@ -143,18 +143,25 @@ extern "C" int hfs_step1d_noalloc(void *psi, int precision, const hfs_instance *
     if (nsteps == 0) return HFS_OK;
 
     // ---- work list: sorted by decreasing N, 256/T instances per item -----
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return HFS_ERR_CUDA;
+    const bool fp64 = precision == HFS_C128;
     for (int64_t i = 0; i < count; ++i) t_order[i] = (int32_t)i;
     std::stable_sort(t_order, t_order + count, [](int32_t x, int32_t y) { return t_inst[x].n[0] > t_inst[y].n[0]; });
+    const bool mixed = t_inst[t_order[0]].n[0] != t_inst[t_order[count - 1]].n[0];
+    const bool small = !fp64 && small1d_ok(t_inst, count, off, sms);
     int32_t nwork = 0;
     for (int64_t i = 0; i < count;) {
         const int n = t_inst[t_order[i]].n[0];
-        const int per = kCtaThreads / (n / 16);
+        const int e = default_ept(n, off, mixed, sms, fp64);
+        const int per = kCtaThreads / (n / e);
         int64_t j = i;
         while (j < count && j - i < per && t_inst[t_order[j]].n[0] == n) ++j;
         t_work[nwork].first = (int32_t)i;
         t_work[nwork].count = (int32_t)(j - i);
-        t_work[nwork].plan = plan_id(n, 16);
-        t_work[nwork].pad = 0;
+        t_work[nwork].plan = t_work[nwork].diag = plan_id(n, e);
         ++nwork;
         i = j;
     }
@@ -165,7 +172,6 @@ extern "C" int hfs_step1d_noalloc(void *psi, int precision, const hfs_instance *
     unsigned char *base = nullptr;
     int s = device_scratch(st, &base);
     if (s) return s;
-    const bool fp64 = precision == HFS_C128;
     unsigned *status = reinterpret_cast<unsigned *>(base + kOffStatus);
     unsigned *ticket = reinterpret_cast<unsigned *>(base + kOffTicket);
     double *tdev = reinterpret_cast<double *>(base + kOffTime);
@@ -182,9 +188,6 @@ extern "C" int hfs_step1d_noalloc(void *psi, int precision, const hfs_instance *
     HFS_NA_CK(cudaMemcpyAsync(base + kOffOrder, t_order, sizeof(int32_t) * count, cudaMemcpyHostToDevice, st));
     HFS_NA_CK(cudaMemcpyAsync(base + kOffWork, t_work, sizeof(WorkItem) * nwork, cudaMemcpyHostToDevice, st));
     HFS_NA_CK(launch_set_time(tdev, t0, st));
-    int dev = 0, sms = 0;
-    HFS_NA_CK(cudaGetDevice(&dev));
-    HFS_NA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int variant = step1d_variant(inst, count);
     const int grid = std::max(1, std::min(nwork, sms * step1d_ctas_per_sm(fp64, variant)));
     for (int64_t done = 0; done < nsteps; done += kNoAllocChunk) {
@@ -209,6 +212,10 @@ extern "C" int hfs_step1d_noalloc(void *psi, int precision, const hfs_instance *
         a.tw = fp64 ? (const void *)(base + kOffTwd) : (const void *)(base + kOffTwf);
         a.ticket = ticket;
         a.status = status;
+        if (small) {
+            HFS_NA_CK(launch_small1d({a, (int32_t)count, 0, sc, tdev, nullptr}, t_inst[t_order[0]].n[0], variant, st));
+            continue;
+        }
         HFS_NA_CK(cudaMemsetAsync(ticket, 0, sizeof(unsigned), st));
         HFS_NA_CK(launch_step1d(fp64, variant, a, grid, st));
     }

@@ -65,6 +65,22 @@ struct Step1DArgs {
     int32_t proj;                   // PROJ_OFF, PROJ_SET (first launch of a call), PROJ_USE
     int32_t streaming;              // fewer sub-stages per launch than the chunk holds (streaming mode)
 };
+// The step kernel of few instances (hfs_step1d_small.cu, complex64): one CTA an
+// instance.  With sched_steps > 0 it computes the records of that many steps
+// from *t_dev itself and the last CTA to finish advances *t_dev (done: a zeroed
+// counter), so that the whole call is one launch.
+struct Small1DArgs {
+    Step1DArgs a;
+    int32_t count, sched_steps;
+    SchedConst sc;
+    double *t_dev;
+    unsigned *done;
+};
+constexpr int kSmallSchedStages = 32;  // sub-stages at most that it computes itself
+// whether a complex64 batch without set plans takes it
+bool small1d_ok(const DevInst *inst, int64_t count, int64_t points, int sms);
+cudaError_t launch_small1d(const Small1DArgs &s, int nmax, int variant, cudaStream_t st, int priority = 0);
+
 enum : int32_t { PROJ_OFF = 0, PROJ_SET = 1, PROJ_USE = 2 };
 // variant: HFS_VI_* when every instance has that perturbation kind and a box
 // symmetric about 0 (FP32 only; from step1d_variant), -1 for the generic kernel
@@ -93,6 +109,10 @@ cudaError_t launch_diag1d(bool fp64, bool energy, const Diag1DArgs &a, int sms, 
 cudaError_t launch_twiddles(void *tw_f, void *tw_d, cudaStream_t st);
 // the plain FP32 table (same layout, the FP64 value rounded to float2)
 cudaError_t launch_twiddles_plain(void *tw_p, cudaStream_t st);
+
+// values per thread of grid size n in a batch without a set plan: points is
+// the batch's total, mixed whether it holds more than one grid size (hfs_api.cu)
+int default_ept(int n, int64_t points, bool mixed, int sms, bool fp64);
 
 // host helpers shared by the entry points (hfs_api.cu)
 int composition_fixed(int comp, double *a, double *b, int *m);

@@ -177,12 +177,12 @@ __global__ void energy_pre_kernel(const Diag1DArgs a)
     const DevInst &ip = a.inst[idx];
     StageFGE r{};
     r.f = 0.5 * ip.mu * law_omega2(ip, *a.t_dev);
-    sincos(ip.vi_k * (ip.dx[0] * (ip.n[0] / plan_ept(it.plan))), &r.e, &r.g);
+    sincos(ip.vi_k * (ip.dx[0] * (ip.n[0] / plan_ept(it.diag))), &r.e, &r.g);
     a.pre[idx] = r;
 }
 
-// items of a batch hold the same number of points each but for the last of a
-// grid size, so CTAs take them in turn
+// items of a batch hold about the same number of points each, so CTAs take them
+// in turn
 template <typename R, bool ENERGY> __global__ void __launch_bounds__(kCtaThreads) diag1d_kernel(const Diag1DArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -190,7 +190,7 @@ template <typename R, bool ENERGY> __global__ void __launch_bounds__(kCtaThreads
     __shared__ double slots[kCtaThreads / 32];
     for (int w = blockIdx.x; w < a.nwork; w += gridDim.x) {
         const WorkItem it = a.work[w];
-        switch (it.plan) {
+        switch (it.diag) {
 #define HFS_CASE(NN, EE, AA)                                                                                      \
     case plan_id(NN, EE, AA):                                                                                     \
         if constexpr (ENERGY) energy_item<R, NN, EE, AA>(a, it, smem, slots);                                      \

@@ -46,6 +46,59 @@ def test_idle_warps(precision, tol, n, count):
     assert _worst(insts, psis, 6, precision) <= budget(tol, 0.03)
 
 
+@pytest.mark.parametrize("sizes,count", [((128,), 1), ((256, 1024), 9), ((2048,), 5), ((128, 512, 4096), 7),
+                                         ((1024,), 152), ((1024,), 153)])
+@pytest.mark.parametrize("project", [False, True])
+@pytest.mark.parametrize("flow,split,scheme", [(0, 0, "strang"), (1, 0, "srkn6_4"), (2, 0, "ni5_84"), (1, 1, "strang")])
+def test_few_instances(sizes, count, project, flow, split, scheme):
+    """The step kernel of few instances against the batch kernel with the same
+    schedule (the same bits without the projection, but for 2048 points): calls whose records it makes itself (up to 32 sub-stages) and
+    longer ones, one launch or one per step (bitwise equal), off-centre boxes and
+    mixed kinds; 152 instances of 1024 points are the most that it takes (153 run in the batch
+    kernel, with another plan than the set one)."""
+    need_gpu()
+    from paper_1007_3470_gb300 import hfs
+    insts, psis, _ = W.batch_1d(count=count, seed=count, sizes=sizes)
+    for k, inst in enumerate(insts):
+        if k % 3 == 1:
+            inst.a[0] += 0.25
+            inst.b[0] += 0.25
+        if k % 3 == 2:
+            inst.vi_kind = W.VI_NONE
+
+    def run(plan, mode=(0, 1), graphs=False):
+        s = hfs.Solver(insts, precision="c64", chunk_steps=24)
+        s.set_schedule(0.01, scheme, flow, split=split)
+        s.set_norm_projection(project)
+        s.set_mode(*mode)
+        if plan:
+            for n in sizes:
+                s.set_plan(n, 16)
+        s.set_graphs(graphs)
+        s.set_psi(psis)
+        for k in (1, 4, 24, 1, 30):
+            s.step(k)
+        out, t = s.get_psi(), s.time
+        norm = s.norm()
+        assert s.status() == hfs.HFS_OK
+        s.close()
+        return out, t, norm
+
+    out, t, norm = run(False)
+    ref, t_ref, _ = run(True)
+    assert t == t_ref
+    # two FP32 solutions of 60 steps to T = 0.6, each within 1e-5 of the exact one
+    assert np.linalg.norm(out - ref) <= 2 * budget(TOL_C64, 0.6) * np.linalg.norm(ref)
+    if not project and 2048 not in sizes and count != 153:
+        assert np.array_equal(out, ref)
+    off = np.concatenate([[0], np.cumsum([i.n[0] for i in insts])])
+    dx = np.array([(i.b[0] - i.a[0]) / i.n[0] for i in insts])
+    sums = dx * np.array([np.sum(np.abs(out[off[k]:off[k + 1]].astype(np.complex128)) ** 2) for k in range(count)])
+    assert np.allclose(norm, sums, rtol=1e-12)
+    assert np.array_equal(out, run(False, mode=(1, 1))[0])
+    assert np.array_equal(out, run(False, graphs=True)[0])
+
+
 @pytest.mark.parametrize("vi", [W.VI_NONE, W.VI_X4, W.VI_COS])
 @pytest.mark.parametrize("shift", [False, True])
 @pytest.mark.parametrize("split", [0, 1])
