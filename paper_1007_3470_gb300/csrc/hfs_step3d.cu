@@ -36,6 +36,18 @@ template <int N> struct Geo3 {
     static constexpr int TX = (kCtaThreads / T < N) ? kCtaThreads / T : N;  // columns per y/z tile
     static constexpr int TT = T * TX;               // threads of a y/z tile CTA
 };
+// The line passes.  FP64 is bound by the FP64 pipe of the SMs that hold a CTA, so
+// the smaller grids are cut into CTAs of one or two warps (64^3 as 64 CTAs of 256
+// // threads left more than half of the SMs idle: 196 us a step of phases and
+// transforms, 107 us now; 32^3 125 us, 48 us now).
+template <typename R, int N> struct LineGeo {
+    static constexpr bool kSmall = sizeof(R) == 8 && N < 128;
+    static constexpr int E = kSmall ? 8 : 16, T = N / E;
+    static constexpr int THREADS = !kSmall ? kCtaThreads : N == 32 ? 32 : 64;
+    static constexpr int G = THREADS / T;
+    static constexpr int TX = G < N ? G : N;
+    static constexpr int TT = T * TX;
+};
 
 __device__ __forceinline__ float turns_q(int m, float hi, float lo) { return frac_turns((float)(m * m), hi, lo); }
 __device__ __forceinline__ double turns_q(int m, double c, double) { return frac_turns((double)m * m, c, 0.0); }
@@ -46,10 +58,10 @@ enum : int { X_INV = 1, X_PHASE = 2, X_FWD = 4 };
 // x-pass
 // ---------------------------------------------------------------------------
 template <typename R, int N, int MODE>
-__global__ void __launch_bounds__(kCtaThreads) xpass3d(const Step3DArgs a, int64_t j)
+__global__ void __launch_bounds__(LineGeo<R, N>::THREADS) xpass3d(const Step3DArgs a, int64_t j)
 {
     using Rec = typename Rec3Of<R>::type;
-    using GEO = Geo3<N>;
+    using GEO = LineGeo<R, N>;
     constexpr int E = GEO::E, T = GEO::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int g = threadIdx.x / T, t = threadIdx.x - g * T;
@@ -64,7 +76,7 @@ __global__ void __launch_bounds__(kCtaThreads) xpass3d(const Step3DArgs a, int64
     if constexpr (MODE & X_PHASE) {
         const DevInst &ip = *a.inst;
         const int vkind = (ip.eps != 0.0) ? ip.vi_kind : HFS_VI_NONE;
-        for (int i = threadIdx.x; i < 3 * N; i += kCtaThreads)
+        for (int i = threadIdx.x; i < 3 * N; i += GEO::THREADS)
             s_v[i / N][i % N] = vi_eval(vkind, (R)(i % N - N / 2) * (R)ip.dx[i / N], (R)ip.vi_k);
         __syncthreads();
     }
@@ -107,9 +119,9 @@ __global__ void __launch_bounds__(kCtaThreads) xpass3d(const Step3DArgs a, int64
 // y-pass: one CTA = fixed z, TX adjacent x columns; lines along y
 // ---------------------------------------------------------------------------
 template <typename R, int N, bool INV>
-__global__ void __launch_bounds__(kCtaThreads) ypass3d(const Step3DArgs a)
+__global__ void __launch_bounds__(LineGeo<R, N>::THREADS) ypass3d(const Step3DArgs a)
 {
-    using GEO = Geo3<N>;
+    using GEO = LineGeo<R, N>;
     constexpr int E = GEO::E, T = GEO::T, TX = GEO::TX;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int l = threadIdx.x % TX, t = threadIdx.x / TX;
@@ -179,10 +191,10 @@ __device__ __forceinline__ void fft3(cpx<R> (&v)[E], cpx<R> *sm, int t, const St
 }
 
 template <typename R, int N, bool PROJ = false>
-__global__ void __launch_bounds__(kCtaThreads, ZpassMinCtas<R>::value) zpass3d(const Step3DArgs a, int64_t j)
+__global__ void __launch_bounds__(LineGeo<R, N>::THREADS, ZpassMinCtas<R>::value) zpass3d(const Step3DArgs a, int64_t j)
 {
     using Rec = typename Rec3Of<R>::type;
-    using GEO = Geo3<N>;
+    using GEO = LineGeo<R, N>;
     constexpr int E = GEO::E, T = GEO::T, TX = GEO::TX;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int l = threadIdx.x % TX, t = threadIdx.x / TX;
@@ -460,6 +472,124 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane3d(const Step3DArgs a, 
 }
 
 // ---------------------------------------------------------------------------
+// complex64, n = 32 and 64: a plane pass and a z-pass per sub-stage, as at 128,
+// with eight values a thread (n^2/8 threads hold a whole plane, one line
+// transform each at a time) and every launch programmatic.  Bound by latency:
+// the state lies in L2 and a pass is one chain of load, transforms and store.
+// Four line passes took 17.8 us a step at 64^3 and 17.8 us at 32^3 (27 us without
+// graph replay); these take 8.3 us and 6.1 us (6.9 us).
+// ---------------------------------------------------------------------------
+template <int N> struct Cube {
+    static constexpr int E = 8, T = N / E, ROW = smem_elems(N);
+    static constexpr int PLANE_THREADS = N * T;
+    static constexpr int TX = 128 / T, Z_THREADS = 128;  // z tile: TX columns
+};
+
+template <int N, int VI, bool FIRST, bool LAST>
+__global__ void __launch_bounds__(Cube<N>::PLANE_THREADS) cube_plane(const Step3DArgs a, int64_t j)
+{
+    constexpr int E = Cube<N>::E, T = Cube<N>::T, ROW = Cube<N>::ROW;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cpx<float> *pl = reinterpret_cast<cpx<float> *>(smem_raw);
+    __shared__ float s_v[2][N];  // eps V_I along x, V_I along y
+    const DevInst &ip = *a.inst;
+    const int z = blockIdx.x;
+    const float vk = (float)ip.vi_k, eps = (float)ip.eps, sig = (float)ip.sigma;
+    for (int i = threadIdx.x; i < 2 * N; i += Cube<N>::PLANE_THREADS) {
+        const int ax = i / N, k = i % N;
+        s_v[ax][k] = (ax == 0 ? eps : 1.0f) * vi_eval(VI, (float)(k - N / 2) * (float)ip.dx[ax], vk);
+    }
+    const float vz = vi_eval(VI, (float)(z - N / 2) * (float)ip.dx[2], vk);
+    const Rec3F rc = reinterpret_cast<const Rec3F *>(a.rec)[j];
+    const float tz = turns_q(z - N / 2, rc.k2[2], rc.k2lo[2]);
+    const float4 *tw = reinterpret_cast<const float4 *>(a.tw);
+    pdl_wait();
+    pdl_trigger();
+    cpx<float> *psi = reinterpret_cast<cpx<float> *>(a.psi) + (int64_t)z * N * N;
+    cpx<float> v[E];
+    const int cx = threadIdx.x % N, ct = threadIdx.x / N;  // column pass: x, thread of the line
+    const int y = threadIdx.x / T, t = threadIdx.x - y * T;  // row pass
+    cpx<float> *col = pl + spad(cx), *row = pl + y * ROW;
+    if constexpr (!FIRST) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = psi[(ct + T * e) * N + cx];
+        FftPlan<N, E>::template run<true, float, ROW>(v, col, ct, tw);
+#pragma unroll
+        for (int e = 0; e < E; ++e) col[(ct + T * e) * ROW] = v[e];
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = row[spad(t + T * e)];
+        __syncwarp();
+        FftPlan<N, E>::template run<true, float, 1, true>(v, row, t, tw);
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = psi[y * N + t + T * e];
+        __syncthreads();  // the table
+    }
+    const float tyz = turns_q(y - N / 2, rc.k2[1], rc.k2lo[1]) + tz;
+    const float evyz = eps * (s_v[1][y] + vz);
+#pragma unroll
+    for (int e = 0; e < E; e += 2) {
+        const int m0 = t + T * e - N / 2, m1 = m0 + T;
+        const Turns2 tx = frac_turns2<true>(make_float2((float)(m0 * m0), (float)(m1 * m1)), rc.k2[0], rc.k2lo[0]);
+        const float d0 = v[e].x * v[e].x + v[e].y * v[e].y, d1 = v[e + 1].x * v[e + 1].x + v[e + 1].y * v[e + 1].y;
+        const float2 F = make_float2(sig * d0 + (s_v[0][m0 + N / 2] + evyz), sig * d1 + (s_v[0][m1 + N / 2] + evyz));
+        apply_turns2(v[e], v[e + 1],
+                     __ffma2_rn(bc2(rc.sb2pi), F, __fadd2_rn(__fadd2_rn(tx.r, tx.c), bc2(tyz))), 1.0f);
+    }
+    if constexpr (LAST) {
+        bool bad = false;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            psi[y * N + t + T * e] = v[e];
+            bad |= !(isfinite(v[e].x) && isfinite(v[e].y));
+        }
+        if (bad) atomicOr(a.status, (unsigned)ST_NONFINITE);
+    } else {
+        FftPlan<N, E>::template run<false, float, 1, true>(v, row, t, tw);
+#pragma unroll
+        for (int e = 0; e < E; ++e) row[spad(t + T * e)] = v[e];
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = col[(ct + T * e) * ROW];
+        __syncthreads();
+        FftPlan<N, E>::template run<false, float, ROW>(v, col, ct, tw);
+#pragma unroll
+        for (int e = 0; e < E; ++e) psi[(ct + T * e) * N + cx] = v[e];
+    }
+}
+
+template <int N> __global__ void __launch_bounds__(Cube<N>::Z_THREADS) cube_z(const Step3DArgs a, int64_t j)
+{
+    constexpr int E = Cube<N>::E, T = Cube<N>::T, TX = Cube<N>::TX;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int l = threadIdx.x % TX, t = threadIdx.x / TX;
+    const int y = blockIdx.y, x = blockIdx.x * TX + l;
+    cpx<float> *sm = reinterpret_cast<cpx<float> *>(smem_raw) + l;
+    cpx<float> *psi = reinterpret_cast<cpx<float> *>(a.psi) + (int64_t)y * N + x;
+    const float4 *tw = reinterpret_cast<const float4 *>(a.tw);
+    const Rec3F rc = reinterpret_cast<const Rec3F *>(a.rec)[j];
+    const int mx = (x < N / 2) ? x : x - N, my = (y < N / 2) ? y : y - N;
+    const float txy = turns_q(mx, rc.g[0], rc.glo[0]) + turns_q(my, rc.g[1], rc.glo[1]);
+    pdl_wait();
+    pdl_trigger();
+    cpx<float> v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = psi[(int64_t)(t + T * e) * N * N];
+    FftPlan<N, E>::template run<false, float, TX>(v, sm, t, tw);
+#pragma unroll
+    for (int e = 0; e < E; e += 2) {
+        const int m0 = t + T * e - (2 * e < E ? 0 : N), m1 = m0 + T;
+        const Turns2 tz = frac_turns2<true>(make_float2((float)(m0 * m0), (float)(m1 * m1)), rc.g[2], rc.glo[2]);
+        apply_turns2(v[e], v[e + 1], __fadd2_rn(bc2(txy), __fadd2_rn(tz.r, tz.c)),
+                     1.0f / ((float)N * (float)N * (float)N));
+    }
+    FftPlan<N, E>::template run<true, float, TX>(v, sm, t, tw);
+#pragma unroll
+    for (int e = 0; e < E; ++e) psi[(int64_t)(t + T * e) * N * N] = v[e];
+}
+
+// ---------------------------------------------------------------------------
 // diagnostics: norm, potential + interaction, and the kinetic energy as a sum
 // over axes of 1D Parseval sums  sum_x |d_d u|^2 = (1/n) sum_k k_d^2 |F_d u|^2
 // ---------------------------------------------------------------------------
@@ -560,12 +690,16 @@ template <typename R, int N, int AXIS> __global__ void __launch_bounds__(kCtaThr
 // ---------------------------------------------------------------------------
 bool step3d_supported(int nx, int ny, int nz) { return nx == ny && ny == nz && (nx == 32 || nx == 64 || nx == 128); }
 
-template <typename R, int N> static size_t xsmem() { return (size_t)Geo3<N>::G * smem_elems(N) * sizeof(cpx<R>); }
-template <typename R, int N> static size_t tsmem()
+// shared memory of the line passes and of the diagnostics
+template <typename R, int N> static size_t xsmem() { return (size_t)LineGeo<R, N>::G * smem_elems(N) * sizeof(cpx<R>); }
+template <typename R, int N> static size_t tsmem() { return (size_t)LineGeo<R, N>::TX * N * sizeof(cpx<R>); }
+template <typename R, int N> static size_t diag_xsmem()
 {
-    const size_t a = (size_t)Geo3<N>::TX * N * sizeof(cpx<R>);
-    const size_t b = 2 * sizeof(double) * Geo3<N>::TT;
-    return a > b ? a : b;
+    return std::max((size_t)Geo3<N>::G * smem_elems(N) * sizeof(cpx<R>), 2 * sizeof(double) * kCtaThreads);
+}
+template <typename R, int N> static size_t diag_tsmem()
+{
+    return std::max((size_t)Geo3<N>::TX * N * sizeof(cpx<R>), 2 * sizeof(double) * Geo3<N>::TT);
 }
 
 template <typename K> static cudaError_t allow_smem(K kernel, size_t bytes)
@@ -593,7 +727,7 @@ static cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
 
 template <typename R, int N> static cudaError_t run3d(const Step3DArgs &a, cudaStream_t st)
 {
-    using GEO = Geo3<N>;
+    using GEO = LineGeo<R, N>;
     const size_t xs = xsmem<R, N>(), ts = tsmem<R, N>();
     static bool prepared = false;
     if (!prepared) {
@@ -609,7 +743,7 @@ template <typename R, int N> static cudaError_t run3d(const Step3DArgs &a, cudaS
         prepared = true;
     }
     const dim3 xg(N * N / GEO::G), tg(N / GEO::TX, N);
-    xpass3d<R, N, X_PHASE | X_FWD><<<xg, kCtaThreads, xs, st>>>(a, 0);
+    xpass3d<R, N, X_PHASE | X_FWD><<<xg, GEO::THREADS, xs, st>>>(a, 0);
     ypass3d<R, N, false><<<tg, GEO::TT, ts, st>>>(a);
     for (int64_t j = 0; j < a.nstage; ++j) {
         if constexpr (sizeof(R) == 4 && (N == 64 || N == 128)) {
@@ -620,10 +754,10 @@ template <typename R, int N> static cudaError_t run3d(const Step3DArgs &a, cudaS
         }
         ypass3d<R, N, true><<<tg, GEO::TT, ts, st>>>(a);
         if (j + 1 < a.nstage) {
-            xpass3d<R, N, X_INV | X_PHASE | X_FWD><<<xg, kCtaThreads, xs, st>>>(a, j + 1);
+            xpass3d<R, N, X_INV | X_PHASE | X_FWD><<<xg, GEO::THREADS, xs, st>>>(a, j + 1);
             ypass3d<R, N, false><<<tg, GEO::TT, ts, st>>>(a);
         } else {
-            xpass3d<R, N, X_INV | X_PHASE><<<xg, kCtaThreads, xs, st>>>(a, j + 1);
+            xpass3d<R, N, X_INV | X_PHASE><<<xg, GEO::THREADS, xs, st>>>(a, j + 1);
         }
     }
     return cudaGetLastError();
@@ -632,11 +766,11 @@ template <typename R, int N> static cudaError_t run3d(const Step3DArgs &a, cudaS
 template <typename R, int N> static cudaError_t diag3d(const Diag3DArgs &a, cudaStream_t st)
 {
     using GEO = Geo3<N>;
-    const size_t xs = xsmem<R, N>(), ts = tsmem<R, N>();
+    const size_t xs = diag_xsmem<R, N>(), ts = diag_tsmem<R, N>();
     static bool prepared = false;
     if (!prepared) {
         cudaError_t e;
-        if ((e = allow_smem(diagx3d<R, N>, std::max(xs, 2 * sizeof(double) * kCtaThreads))) != cudaSuccess) return e;
+        if ((e = allow_smem(diagx3d<R, N>, xs)) != cudaSuccess) return e;
         if ((e = allow_smem(diagyz3d<R, N, 1>, ts)) != cudaSuccess) return e;
         if ((e = allow_smem(diagyz3d<R, N, 2>, ts)) != cudaSuccess) return e;
         prepared = true;
@@ -644,10 +778,36 @@ template <typename R, int N> static cudaError_t diag3d(const Diag3DArgs &a, cuda
     cudaError_t e = cudaMemsetAsync(a.out, 0, 2 * sizeof(double), st);
     if (e != cudaSuccess) return e;
     const dim3 xg(N * N / GEO::G), tg(N / GEO::TX, N);
-    diagx3d<R, N><<<xg, kCtaThreads, std::max(xs, 2 * sizeof(double) * kCtaThreads), st>>>(a);
+    diagx3d<R, N><<<xg, kCtaThreads, xs, st>>>(a);
     diagyz3d<R, N, 1><<<tg, GEO::TT, ts, st>>>(a);
     diagyz3d<R, N, 2><<<tg, GEO::TT, ts, st>>>(a);
     return cudaGetLastError();
+}
+
+template <int N, int VI> static cudaError_t run3d_cube_vi(const Step3DArgs &a, cudaStream_t st)
+{
+    using C = Cube<N>;
+    const size_t ps = (size_t)N * C::ROW * sizeof(cpx<float>), zs = (size_t)C::TX * N * sizeof(cpx<float>);
+    const dim3 zg(N / C::TX, N);
+    // as run3d_plane_vi: the first pass follows the records in plain stream order
+    cube_plane<N, VI, true, false><<<N, C::PLANE_THREADS, ps, st>>>(a, 0);
+    cudaError_t e = cudaGetLastError();
+    for (int64_t j = 0; j < a.nstage && e == cudaSuccess; ++j) {
+        e = launch_pdl(cube_z<N>, zg, dim3(C::Z_THREADS), zs, st, a, j);
+        if (e != cudaSuccess) break;
+        if (j + 1 < a.nstage) e = launch_pdl(cube_plane<N, VI, false, false>, dim3(N), dim3(C::PLANE_THREADS), ps, st, a, j + 1);
+        else e = launch_pdl(cube_plane<N, VI, false, true>, dim3(N), dim3(C::PLANE_THREADS), ps, st, a, j + 1);
+    }
+    return e;
+}
+template <int N> static cudaError_t run3d_cube(const Step3DArgs &a, cudaStream_t st)
+{
+    switch (a.vi) {
+    case HFS_VI_COS: return run3d_cube_vi<N, HFS_VI_COS>(a, st);
+    case HFS_VI_X4: return run3d_cube_vi<N, HFS_VI_X4>(a, st);
+    case HFS_VI_NONE: return run3d_cube_vi<N, HFS_VI_NONE>(a, st);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 template <int VI, bool PROJ> static cudaError_t run3d_plane_vi(const Step3DArgs &a, cudaStream_t st)
@@ -698,9 +858,9 @@ cudaError_t launch_step3d(bool fp64, const Step3DArgs &a, cudaStream_t st)
 {
     if (!fp64 && a.n == kPlaneN) return run3d_plane(a, st);
     switch (a.n) {
-    case 32: return fp64 ? run3d<double, 32>(a, st) : run3d<float, 32>(a, st);
-    case 64: return fp64 ? run3d<double, 64>(a, st) : run3d<float, 64>(a, st);
-    case 128: return fp64 ? run3d<double, 128>(a, st) : run3d<float, 128>(a, st);
+    case 32: return fp64 ? run3d<double, 32>(a, st) : run3d_cube<32>(a, st);
+    case 64: return fp64 ? run3d<double, 64>(a, st) : a.dft_tc ? run3d<float, 64>(a, st) : run3d_cube<64>(a, st);
+    case 128: return fp64 ? run3d<double, 128>(a, st) : cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
     }
 }
