@@ -139,7 +139,8 @@ struct hfs_ctx_s {
     bool law_shared = false;
     // specialised 1D step kernel (step1d_variant), -1 for the generic one
     int variant = -1;
-    bool small = false;  // few complex64 instances without set plans (small1d_ok)
+    // few instances without set plans: small1d_ok (complex64), cluster1d_ok (complex128)
+    bool small = false, cluster = false;
     std::vector<int32_t> order;  // sorted position -> instance
     std::vector<WorkItem> work;
     // schedule
@@ -249,7 +250,9 @@ void build_worklist(hfs_ctx_s *c)
                      [&](int32_t x, int32_t y) { return c->inst[x].n[0] > c->inst[y].n[0]; });
     c->work.clear();
     c->small = c->precision == HFS_C64 && small1d_ok(c->dinst.data(), c->count, c->elems, c->sm_count);
-    for (auto &p : c->inst) c->small = c->small && !c->plan_set[size_class(p.n[0])];
+    c->cluster = c->precision == HFS_C128 && cluster1d_ok(c->dinst.data(), c->count, c->sm_count);
+    for (auto &p : c->inst)
+        if (c->plan_set[size_class(p.n[0])]) c->small = c->cluster = false;
     const bool fp64 = c->precision == HFS_C128, mixed = c->inst[c->order[0]].n[0] != c->inst[c->order[c->count - 1]].n[0];
     int64_t i = 0;
     while (i < c->count) {
@@ -450,6 +453,10 @@ int enqueue_steps(hfs_ctx_s *c, int64_t nsteps, const ReusePlan &rp = ReusePlan(
                 if (c->small) {
                     const Small1DArgs sa{a, (int32_t)c->count, own ? (int32_t)S : 0, c->sc, tdev, ticket + 1};
                     CK(launch_small1d(sa, c->inst[c->order[0]].n[0], c->variant, c->stream, rp.prefetch ? c->prio_high : 0));
+                    continue;
+                }
+                if (c->cluster) {
+                    CK(launch_cluster1d(a, c->inst[0].n[0], (int)c->count, c->stream, rp.prefetch ? c->prio_high : 0));
                     continue;
                 }
                 CK(cudaMemsetAsync(ticket, 0, sizeof(unsigned), c->stream));

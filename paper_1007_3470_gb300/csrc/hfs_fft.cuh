@@ -496,6 +496,10 @@ HFS_PLAN(1024, 4, 4, 4, 4, 4, 4)
 HFS_PLAN(512, 4, 4, 4, 4, 4, 2)
 HFS_PLAN(256, 4, 4, 4, 4, 4)
 HFS_PLAN(128, 4, 4, 4, 4, 2)
+// the factors of a transform spread over a cluster (hfs_step1d_cluster.cu)
+HFS_PLAN(64, 4, 4, 4, 4)
+HFS_PLAN(32, 4, 4, 4, 2)
+HFS_PLAN(16, 4, 4, 4)
 // sixteen values per thread, alternative radix orders
 HFS_PLAN_ORDER(4096, 16, true, 8, 8, 8, 8)
 HFS_PLAN_ORDER(2048, 16, true, 8, 16, 16)

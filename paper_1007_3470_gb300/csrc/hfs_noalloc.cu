@@ -152,6 +152,7 @@ extern "C" int hfs_step1d_noalloc(void *psi, int precision, const hfs_instance *
     std::stable_sort(t_order, t_order + count, [](int32_t x, int32_t y) { return t_inst[x].n[0] > t_inst[y].n[0]; });
     const bool mixed = t_inst[t_order[0]].n[0] != t_inst[t_order[count - 1]].n[0];
     const bool small = !fp64 && small1d_ok(t_inst, count, off, sms);
+    const bool cluster = fp64 && cluster1d_ok(t_inst, count, sms);
     int32_t nwork = 0;
     for (int64_t i = 0; i < count;) {
         const int n = t_inst[t_order[i]].n[0];
@@ -214,6 +215,10 @@ extern "C" int hfs_step1d_noalloc(void *psi, int precision, const hfs_instance *
         a.status = status;
         if (small) {
             HFS_NA_CK(launch_small1d({a, (int32_t)count, 0, sc, tdev, nullptr}, t_inst[t_order[0]].n[0], variant, st));
+            continue;
+        }
+        if (cluster) {
+            HFS_NA_CK(launch_cluster1d(a, t_inst[0].n[0], (int)count, st));
             continue;
         }
         HFS_NA_CK(cudaMemsetAsync(ticket, 0, sizeof(unsigned), st));

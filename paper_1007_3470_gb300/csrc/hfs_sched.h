@@ -81,6 +81,11 @@ constexpr int kSmallSchedStages = 32;  // sub-stages at most that it computes it
 bool small1d_ok(const DevInst *inst, int64_t count, int64_t points, int sms);
 cudaError_t launch_small1d(const Small1DArgs &s, int nmax, int variant, cudaStream_t st, int priority = 0);
 
+// The step kernel of few complex128 instances of one grid size
+// (hfs_step1d_cluster.cu): one cluster an instance.
+bool cluster1d_ok(const DevInst *inst, int64_t count, int sms);
+cudaError_t launch_cluster1d(const Step1DArgs &a, int n, int count, cudaStream_t st, int priority = 0);
+
 enum : int32_t { PROJ_OFF = 0, PROJ_SET = 1, PROJ_USE = 2 };
 // variant: HFS_VI_* when every instance has that perturbation kind and a box
 // symmetric about 0 (FP32 only; from step1d_variant), -1 for the generic kernel
