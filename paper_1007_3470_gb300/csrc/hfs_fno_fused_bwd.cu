@@ -132,30 +132,38 @@ __global__ void __launch_bounds__(kThreads) head_bwd_kernel(const HeadBwdArgs a)
                 zs[i] = r < valid ? *reinterpret_cast<const float2 *>(a.Qpre + (r0 + r) * P + col) : make_float2(0.0f, 0.0f);
             }
 #pragma unroll 1
-            for (int i = 0; i < 8; ++i) {
-                const int r = r8 + i * groups;
-                if (r >= kHeadRows) break;
-                float2 z = zs[0];
+            for (int i = 0; i < 8; i += 2) {  // two rows' chains of erff and expf side by side
+                if (r8 + i * groups >= kHeadRows) break;
+                float e[4], v[2], q[4];
+                const float z[4] = {zs[0].x, zs[0].y, zs[1].x, zs[1].y};
 #pragma unroll
-                for (int q = 0; q < 7; ++q) zs[q] = zs[q + 1];
-                const float e0 = 1.0f + erff(z.x * 0.70710678118654752f), e1 = 1.0f + erff(z.y * 0.70710678118654752f);
-                const float q0 = __bfloat162float(__float2bfloat16(0.5f * z.x * e0));
-                const float q1 = __bfloat162float(__float2bfloat16(0.5f * z.y * e1));
-                // dO is zero in rows past the end, and with it their dQ and sums
-                float v0 = 0.0f, v1 = 0.0f;
+                for (int k = 0; k < 6; ++k) zs[k] = zs[k + 2];
 #pragma unroll
-                for (int o = 0; o < OCM; ++o) {
-                    const float d = dOs[r * 8 + o];
-                    v0 = fmaf(d, p2[0][o], v0);
-                    v1 = fmaf(d, p2[1][o], v1);
-                    gp2[0][o] = fmaf(q0, d, gp2[0][o]);
-                    gp2[1][o] = fmaf(q1, d, gp2[1][o]);
+                for (int k = 0; k < 4; ++k) {
+                    e[k] = 1.0f + erff(z[k] * 0.70710678118654752f);
+                    q[k] = __bfloat162float(__float2bfloat16(0.5f * z[k] * e[k]));
+                    e[k] = 0.5f * e[k] + z[k] * expf(-0.5f * z[k] * z[k]) * 0.39894228040143268f;
                 }
-                v0 *= 0.5f * e0 + z.x * expf(-0.5f * z.x * z.x) * 0.39894228040143268f;
-                v1 *= 0.5f * e1 + z.y * expf(-0.5f * z.y * z.y) * 0.39894228040143268f;
-                gc1[0] += v0;
-                gc1[1] += v1;
-                *reinterpret_cast<unsigned *>(Qs + tile_at(r, col >> 3, lgP) + (col & 7)) = pack2(v0, v1);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int r = r8 + (i + h) * groups;
+                    if (r >= kHeadRows) break;
+                    // dO is zero in rows past the end, and with it their dQ and sums
+                    v[0] = v[1] = 0.0f;
+#pragma unroll
+                    for (int o = 0; o < OCM; ++o) {
+                        const float d = dOs[r * 8 + o];
+                        v[0] = fmaf(d, p2[0][o], v[0]);
+                        v[1] = fmaf(d, p2[1][o], v[1]);
+                        gp2[0][o] = fmaf(q[2 * h], d, gp2[0][o]);
+                        gp2[1][o] = fmaf(q[2 * h + 1], d, gp2[1][o]);
+                    }
+                    v[0] *= e[2 * h];
+                    v[1] *= e[2 * h + 1];
+                    gc1[0] += v[0];
+                    gc1[1] += v[1];
+                    *reinterpret_cast<unsigned *>(Qs + tile_at(r, col >> 3, lgP) + (col & 7)) = pack2(v[0], v[1]);
+                }
             }
         }
         cp_wait_all();
