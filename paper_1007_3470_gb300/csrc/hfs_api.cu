@@ -72,18 +72,19 @@ int composition_fixed(int comp, double *a, double *b, int *m)
     }
 }
 
-// Values per thread where no plan was set (batches that small1d_ok leaves).  16
-// for large batches of one size, but for 512 points (three radix-8 passes: 11.5
-// against 12.6 us a step of 4096 instances).  8, on twice the threads, while these
-// make at most two 256-thread CTAs an SM (608 instances of 1024 points 4.05
-// against 4.78 us a step, 1216 of them 7.7 against 6.7), and for the sizes up to
-// 1024 of a mixed batch: their shorter, more numerous warps fill the gaps that
-// the long transforms' exchanges leave (4096 instances of 128 ... 4096 points, 200
-// steps: 7.64 -> 7.05 ms, 6.21 -> 5.93 ms with the norm projection).  FP64: 8 until
-// the FP64 pipe has eight warps an SM (one instance of 1024 points: 63 -> 35 us a
-// sub-stage).
-int default_ept(int n, int64_t points, bool mixed, int sms, bool fp64)
+// Values per thread where no plan was set (batches that small1d_ok and
+// cluster1d_ok leave).  FP32 with the norm projection (plain twiddles): 16; 8
+// measured 1 to 5 % slower at 300 to 2000 instances, and rounds in one more pass.
+// FP32 without it: 8, on twice the threads, while these make at most two
+// 256-thread CTAs an SM (608 instances of 1024 points 4.05 against 4.78 us a step,
+// 1216 of them 7.7 against 6.7), at 512 points (three radix-8 passes; 3000
+// instances, 50 steps: 429 against 522 us) and for the sizes up to 1024 of a mixed
+// batch: their shorter, more numerous warps fill the gaps that the long
+// transforms' exchanges leave (4096 instances of 128 ... 4096 points, 60 steps:
+// 2.37 -> 2.20 ms).  FP64: 8 until the FP64 pipe has eight warps an SM.
+int default_ept(int n, int64_t points, bool mixed, bool proj, int sms, bool fp64)
 {
+    if (!fp64 && proj) return 16;
     if (n <= 2048 && points / 8 <= (int64_t)sms * kCtaThreads * (fp64 ? 1 : 2)) return 8;
     if (!fp64 && n <= 1024 && (mixed || n == 512)) return 8;
     return 16;
@@ -258,7 +259,7 @@ void build_worklist(hfs_ctx_s *c)
     while (i < c->count) {
         const int n = c->inst[c->order[i]].n[0];
         const bool set = c->plan_set[size_class(n)], alt = set && c->alt[size_class(n)];
-        const int e = set ? c->ept[size_class(n)] : default_ept(n, c->elems, mixed, c->sm_count, fp64);
+        const int e = set ? c->ept[size_class(n)] : default_ept(n, c->elems, mixed, c->norm_projection, c->sm_count, fp64);
         const int per = kCtaThreads / (n / e);
         int64_t j = i;
         while (j < c->count && j - i < per && c->inst[c->order[j]].n[0] == n) ++j;
@@ -757,6 +758,10 @@ int hfs_set_norm_projection(hfs_ctx_t c, int enable)
     if (c->dim == 3 && c->inst[0].n[0] != 128) return HFS_ERR_UNSUPPORTED;
     c->norm_projection = enable != 0;
     drop_graphs(c);
+    if (c->dim == 1) {  // default plans depend on it
+        build_worklist(c);
+        if (c->work_base) return upload_tables(c);
+    }
     return HFS_OK;
 }
 

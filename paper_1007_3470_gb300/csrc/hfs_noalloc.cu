@@ -156,7 +156,7 @@ extern "C" int hfs_step1d_noalloc(void *psi, int precision, const hfs_instance *
     int32_t nwork = 0;
     for (int64_t i = 0; i < count;) {
         const int n = t_inst[t_order[i]].n[0];
-        const int e = default_ept(n, off, mixed, sms, fp64);
+        const int e = default_ept(n, off, mixed, false, sms, fp64);
         const int per = kCtaThreads / (n / e);
         int64_t j = i;
         while (j < count && j - i < per && t_inst[t_order[j]].n[0] == n) ++j;

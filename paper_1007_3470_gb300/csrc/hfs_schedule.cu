@@ -59,7 +59,7 @@ __global__ void law_nodes_kernel(const DevInst *__restrict__ inst, SchedConst sc
 // and entries in one line (with an integer division each; one block of 128 for
 // every instance left 127 threads idle on calls of one step: 65 + 45 us for
 // 16384 instances).
-constexpr int kFlatBelow = 64;
+constexpr int kFlatBelow = 16;
 struct ItemAt {
     int64_t i;
     int n, stride;  // stride 0: none of this thread's

@@ -392,11 +392,13 @@ __device__ __forceinline__ void step_item(const Step1DArgs &a, const WorkItem &i
     const int g = threadIdx.x / T;
     const int t = threadIdx.x - g * T;
     const bool active = g < it.count;
-    // a warp without an instance leaves the FP32 and FP64 pipes to the others
-    // (one FP64 instance of 1024 points took 201 us a sub-stage with the three
-    // idle teams of its CTA transforming zeros and the longer phases, 63 us
-    // without; one FP32 instance of 256 points 2.7 us a step, 1.9 us without)
-    if ((threadIdx.x & ~31) / T >= it.count) return;
+    // FP64: a warp without an instance leaves the FP64 pipe to the others (one
+    // instance of 1024 points took 201 us a sub-stage with the three idle teams of
+    // its CTA transforming zeros and the longer phases, 63 us without).  FP32: few
+    // instances run in small1d_kernel; the test here cost a full batch 1.6 %.
+    if constexpr (sizeof(R) == 8) {
+        if ((threadIdx.x & ~31) / T >= it.count) return;
+    }
     const int idx = a.order[it.first + (active ? g : 0)];
     const DevInst &ip = a.inst[idx];
     const TeamParams<R> tp = team_params<R>(ip);
