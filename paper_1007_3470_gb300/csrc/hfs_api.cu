@@ -759,8 +759,13 @@ int hfs_set_norm_projection(hfs_ctx_t c, int enable)
     c->norm_projection = enable != 0;
     drop_graphs(c);
     if (c->dim == 1) {  // default plans depend on it
+        const std::vector<WorkItem> old = c->work;
         build_worklist(c);
-        if (c->work_base) return upload_tables(c);
+        const bool same = old.size() == c->work.size() &&
+                          std::equal(old.begin(), old.end(), c->work.begin(), [](const WorkItem &x, const WorkItem &y) {
+                              return x.first == y.first && x.count == y.count && x.plan == y.plan && x.diag == y.diag;
+                          });
+        if (c->work_base && !same) return upload_tables(c);
     }
     return HFS_OK;
 }

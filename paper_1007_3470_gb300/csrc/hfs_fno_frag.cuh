@@ -253,7 +253,10 @@ inline cudaError_t launch_k(void (*kernel)(P...), dim3 grid, int threads, size_t
 
 // CTAs of a persistent grid: as many as fit.  Asked once for a kernel, its
 // shared memory and a device; the slot is the launch site's own, and a race of
-// two threads on it only asks twice.
+// two threads on it only asks twice.  Every kernel is allowed the most shared
+// memory that a CTA may have (none has static arrays), whatever its launch
+// takes, so that models of different sizes do not undo each other's setting.
+constexpr int kMaxSmem = 227 * 1024;
 struct ResidentSlot {
     std::atomic<uint64_t> dev[16];  // (shared memory + 1) << 24 | CTAs
 };
@@ -271,7 +274,7 @@ inline cudaError_t resident_ctas(ResidentSlot &slot, K kernel, int threads, size
             return cudaSuccess;
         }
     }
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
     int sms = 0, per = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
