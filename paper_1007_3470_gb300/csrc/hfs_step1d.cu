@@ -23,11 +23,8 @@ HFS_STEP1D_VARIANT(extern, float, HFS_VI_COS, true)
 // ---------------------------------------------------------------------------
 // the sum over a team's threads (teams of T threads are aligned): in shuffles,
 // then the team's warps through slots
-template <int T> __device__ __forceinline__ double team_sum(double s, double *slots)
+template <int T> __device__ __forceinline__ double team_warps(double s, double *slots)
 {
-    constexpr int W = T < 32 ? T : 32;
-#pragma unroll
-    for (int o = W / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if constexpr (T > 32) {
         const int bar = 1 + threadIdx.x / T, w0 = (threadIdx.x / T) * (T / 32);
         exchange_sync<T, true>(bar);
@@ -39,9 +36,69 @@ template <int T> __device__ __forceinline__ double team_sum(double s, double *sl
     }
     return s;
 }
+template <int T> __device__ __forceinline__ double team_sum(double s, double *slots)
+{
+    constexpr int W = T < 32 ? T : 32;
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return team_warps<T>(s, slots);
+}
 
-// Norm alone: one pass over the state, bound by the FP64 pipe (two FMAs and two
-// conversions a point at 2 lanes a cycle) a little above the memory time.
+// Unevaluated FP32 sums hi + lo.  The FP64 pipe takes 16 cycles a warp
+// instruction, an FP32 instruction a quarter of one (an SM), so sums over an FP32
+// state are formed in two or three floats with exact products and additions
+// (Dekker, Knuth), and only a thread's total enters FP64.
+struct Pair {
+    float hi, lo;
+};
+__device__ __forceinline__ Pair two_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ Pair quick_sum(float a, float b)  // |a| >= |b|
+{
+    const float s = __fadd_rn(a, b);
+    return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ Pair two_prod(float a, float b)
+{
+    const float p = __fmul_rn(a, b);
+    return {p, __fmaf_rn(a, b, -p)};
+}
+__device__ __forceinline__ Pair add(Pair a, Pair b)
+{
+    const Pair s = two_sum(a.hi, b.hi);
+    return quick_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+}
+__device__ __forceinline__ Pair mul(Pair a, Pair b)
+{
+    const Pair p = two_prod(a.hi, b.hi);
+    return quick_sum(p.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo)));
+}
+__device__ __forceinline__ Pair abs2(cpx<float> v)
+{
+    const Pair x = two_prod(v.x, v.x), y = two_prod(v.y, v.y), s = two_sum(x.hi, y.hi);
+    return quick_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(x.lo, y.lo)));
+}
+__device__ __forceinline__ Pair to_pair(double a)
+{
+    const float h = (float)a;
+    return {h, (float)(a - (double)h)};
+}
+template <int T> __device__ __forceinline__ double team_sum(Pair s, double *slots)
+{
+    constexpr int W = T < 32 ? T : 32;
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1)
+        s = add(s, Pair{__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)});
+    return team_warps<T>((double)s.hi + (double)s.lo, slots);
+}
+
+// Norm alone: one pass over the state.  With two FMAs and two conversions a point
+// the FP64 pipe bounds it (a complex128 state's still); an FP32 state's squares
+// are summed exactly in three floats (to 2^-72), 44 FP32 instructions a point.
+// Squares outside FP32's range, or not finite, are summed again in FP64.
 template <typename R, int T, int E>
 __device__ __forceinline__ void norm_item(const Diag1DArgs &a, const WorkItem &it, double *slots)
 {
@@ -51,42 +108,153 @@ __device__ __forceinline__ void norm_item(const Diag1DArgs &a, const WorkItem &i
     const DevInst &ip = a.inst[idx];
     const cpx<R> *psi = reinterpret_cast<const cpx<R> *>(a.psi) + ip.off;
     double s = 0.0;
-    if (active) {
+    bool done = false;
+    if constexpr (sizeof(R) == 4) {
         cpx<R> v[E];
 #pragma unroll
-        for (int e = 0; e < E; ++e) v[e] = psi[t + T * e];
+        for (int e = 0; e < E; ++e) v[e] = active ? psi[t + T * e] : cpx<R>{R(0), R(0)};
+        float hi = 0.0f, mid = 0.0f, lo = 0.0f;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            const double x = v[e].x, y = v[e].y;
+            const Pair x = two_prod(v[e].x, v[e].x), y = two_prod(v[e].y, v[e].y);
+            const Pair d = two_sum(x.hi, y.hi), r = two_sum(x.lo, y.lo);
+            const Pair h = two_sum(hi, d.hi);
+            const Pair m0 = two_sum(mid, h.lo), m1 = two_sum(m0.hi, d.lo), m2 = two_sum(m1.hi, r.hi);
+            hi = h.hi;
+            mid = m2.hi;
+            lo += (m0.lo + m1.lo) + (m2.lo + r.lo);
+        }
+        s = team_sum<T>((double)hi + ((double)mid + (double)lo), slots);
+        done = !active || (s > 1e-18 && s < 1e30);
+        if constexpr (T < 32) done = __all_sync(0xffffffffu, done);
+    }
+    if (!done) {
+        s = 0.0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const cpx<R> u = active ? psi[t + T * e] : cpx<R>{R(0), R(0)};
+            const double x = u.x, y = u.y;
             s = fma(x, x, fma(y, y, s));
         }
+        s = team_sum<T>(s, slots);
     }
-    s = team_sum<T>(s, slots);
     if (active && t == 0) a.out[2 * idx] = s * ip.dx[0];
 }
 
-// FP32 pairs hi + lo: sum += m2 |v|^2, every product and the sum exact to 2^-48
-struct Sum2 {
-    float hi = 0.0f, lo = 0.0f;
-};
-__device__ __forceinline__ void add_m2_abs2(Sum2 &s, float m2, cpx<float> v)
+// The potential's sum over a thread's points in FP64: eight FP64 instructions a
+// point, cos k x by c_{e+1} = 2 cos(k T dx) c_e - c_{e-1} (its error of some E^2
+// roundings is far below the transform's).  c2 = mu omega^2 / 2; g, sg = cos, sin
+// of k T dx.
+template <int N, int E>
+__device__ __forceinline__ double potential_fp64(const DevInst &ip, const cpx<double> (&v)[E], int t, double c2, double g, double sg)
 {
-    const float p = v.x * v.x, q = v.y * v.y;
-    const float pq = p + q, bb = pq - p;
-    const float lo = (p - (pq - bb)) + (q - bb) + fmaf(v.x, v.x, -p) + fmaf(v.y, v.y, -q);
-    const float t = m2 * pq;
-    const float tl = fmaf(m2, lo, fmaf(m2, pq, -t));
-    const float h = s.hi + t, hb = h - s.hi;
-    s.lo += (s.hi - (h - hb)) + (t - hb) + tl;
-    s.hi = h;
+    constexpr int T = N / E;
+    const double hs = 0.5 * ip.sigma, step = T * ip.dx[0];
+    const int kind = ip.eps != 0.0 ? ip.vi_kind : HFS_VI_NONE;
+    double x = ip.xc[0] + (double)(t - N / 2) * ip.dx[0];
+    double pot = 0.0, c = 0.0, cn = 0.0, f = 0.0;
+    if (kind == HFS_VI_COS) {
+        double sn, cs;
+        sincos(ip.vi_k * x, &sn, &cs);
+        f = 2.0 * g;
+        c = ip.eps * cs;
+        cn = ip.eps * (cs * g - sn * sg);
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const double vx = v[e].x, vy = v[e].y;
+        const double d = fma(vx, vx, vy * vy), xx = x * x;
+        double w = fma(hs, d, c2 * xx);
+        if (kind == HFS_VI_COS) {
+            w += c;
+            const double next = fma(f, cn, -c);
+            c = cn;
+            cn = next;
+        } else if (kind == HFS_VI_X4) {
+            w = fma(ip.eps * xx, xx, w);
+        }
+        pot = fma(w, d, pot);
+        x += step;
+    }
+    return pot;
 }
 
-// Energy.  Bound by the FP64 pipe: the potential's sum takes eight FP64
-// instructions a point (cos k x by c_{e+1} = 2 cos(k T dx) c_e - c_{e-1} over the
-// thread's points instead of cos; its error of some E^2 roundings is far below
-// the transform's), the kinetic sum of an FP32 state is formed in FP32 pairs.
-// 4096 mixed-size FP32 instances: norm and energy took 1.19 ms together (0.32 ms
-// now, copies included) as two runs of one kernel with cos and all sums in FP64.
+// What the FP32 energy needs of an instance, in units of the mesh: x = (m + r) dx,
+// the trap as a m^2, eps V_I as b m^4 or cos, sin of k T dx.  a.hi is NaN where a
+// parameter is outside the range of the pairs (the instance is summed in FP64).
+struct alignas(16) EnergyPre {
+    Pair r, a, b, e;
+};
+static_assert(sizeof(EnergyPre) == sizeof(StageFGE), "one record per instance");
+
+// The same sum of an FP32 state in pairs (products and sums to 2^-46, against
+// 1e-8 of the transform), about 100 FP32 instructions a point and FP64 only for
+// the first cosines.  One copy of the code for all plans, reading the points from
+// memory: unrolled over registers it spilled, and its fetch cost more than its
+// issue.
+__device__ __noinline__ Pair potential_pairs(const DevInst &ip, const EnergyPre &pre, const cpx<float> *psi, int t, int T, int E)
+{
+    const Pair hs = to_pair(0.5 * ip.sigma);
+    const int kind = ip.vi_kind_eff, n = T * E;
+    Pair c{}, cn{};
+    if (kind == HFS_VI_COS) {
+        const double g = (double)pre.b.hi + (double)pre.b.lo, sg = (double)pre.e.hi + (double)pre.e.lo;
+        double sn, cs;
+        sincos(ip.vi_k * (ip.xc[0] + (double)(t - n / 2) * ip.dx[0]), &sn, &cs);
+        c = to_pair(ip.eps * cs);
+        cn = to_pair(ip.eps * (cs * g - sn * sg));
+    }
+    const Pair r = pre.r, a = pre.a, b = pre.b, f{2.0f * b.hi, 2.0f * b.lo};
+    Pair pot{};
+    float den = 0.0f;
+#pragma unroll 1
+    for (int e0 = 0; e0 < E; e0 += 4) {
+        cpx<float> v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = psi[t + T * (e0 + e)];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const Pair m = two_sum((float)(t - n / 2 + T * (e0 + e)), r.hi), x = quick_sum(m.hi, m.lo + r.lo);
+            const Pair xx = mul(x, x), d = abs2(v[e]);
+            Pair w = add(mul(a, xx), mul(hs, d));
+            if (kind == HFS_VI_COS) {
+                w = add(w, c);
+                const Pair p = mul(f, cn), next = add(p, Pair{-c.hi, -c.lo});
+                c = cn;
+                cn = next;
+            } else if (kind == HFS_VI_X4) {
+                w = add(w, mul(b, mul(xx, xx)));
+            }
+            pot = add(pot, mul(w, d));
+            den += d.hi;
+        }
+    }
+    if (!(den < 1e6f)) pot.hi = __int_as_float(0x7fffffff);
+    return pot;
+}
+// and in FP64 for a state that the pairs do not hold
+__device__ __noinline__ double potential_wide(const DevInst &ip, double now, const cpx<float> *psi, int t, int T, int E)
+{
+    const double c2 = 0.5 * ip.mu * law_omega2(ip, now);
+    double pot = 0.0;
+#pragma unroll 1
+    for (int e = 0; e < E; ++e) {
+        const int j = t + T * e;
+        const double x = ip.xc[0] + (double)(j - T * E / 2) * ip.dx[0], vx = psi[j].x, vy = psi[j].y;
+        const double d = fma(vx, vx, vy * vy), xx = x * x;
+        double w = fma(0.5 * ip.sigma, d, c2 * xx);
+        if (ip.vi_kind_eff == HFS_VI_COS) w = fma(ip.eps, cos(ip.vi_k * x), w);
+        if (ip.vi_kind_eff == HFS_VI_X4) w = fma(ip.eps * xx, xx, w);
+        pot = fma(w, d, pot);
+    }
+    return pot;
+}
+
+// Energy.  4096 mixed-size FP32 instances: norm and energy took 1.19 ms together
+// (copies included) as two runs of one kernel with cos and all sums in FP64,
+// 0.32 ms with cos by recurrence and the kinetic sum in pairs, which left the FP64
+// pipe 62 % (energy) and 80 % (norm) busy; 0.19 ms with every sum of an FP32 state
+// in floats and two CTAs an SM (128 registers; FP64 sums over registers took 255).
 template <typename R, int N, int E, bool ALT>
 __device__ __forceinline__ void energy_item(const Diag1DArgs &a, const WorkItem &it, cpx<R> *smem, double *slots)
 {
@@ -100,90 +268,99 @@ __device__ __forceinline__ void energy_item(const Diag1DArgs &a, const WorkItem 
     const cpx<R> *psi = reinterpret_cast<const cpx<R> *>(a.psi) + ip.off;
     cpx<R> *sm = smem + g * smem_elems(N);
     const auto *tw = reinterpret_cast<const typename TwOf<R>::type *>(a.tw);
-    cpx<R> v[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) v[e] = active ? psi[t + T * e] : cpx<R>{R(0), R(0)};
-    double pot = 0.0;
-    if (active) {
-        const StageFGE pre = a.pre[idx];
-        const double c2 = pre.f, hs = 0.5 * ip.sigma, step = T * ip.dx[0];
-        const int kind = ip.eps != 0.0 ? ip.vi_kind : HFS_VI_NONE;
-        double x = ip.xc[0] + (double)(t - N / 2) * ip.dx[0];
-        double c = 0.0, cn = 0.0, f = 0.0;
-        if (kind == HFS_VI_COS) {
-            double sn, cs;
-            sincos(ip.vi_k * x, &sn, &cs);
-            f = 2.0 * pre.g;
-            c = ip.eps * cs;
-            cn = ip.eps * (cs * pre.g - sn * pre.e);
-        }
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const double vx = v[e].x, vy = v[e].y;
-            const double d = fma(vx, vx, vy * vy), xx = x * x;
-            double w = fma(hs, d, c2 * xx);
-            if (kind == HFS_VI_COS) {
-                w += c;
-                const double next = fma(f, cn, -c);
-                c = cn;
-                cn = next;
-            } else if (kind == HFS_VI_X4) {
-                w = fma(ip.eps * xx, xx, w);
-            }
-            pot = fma(w, d, pot);
-            x += step;
-        }
-    }
-    FftPlan<N, E, ALT>::template run<false, R, 1, true>(v, sm, t, tw, 1 + g);
     const double ku = 2.0 * 3.14159265358979323846 / ip.len[0], ck = ku * ku / N / (2.0 * ip.mu);
-    bool pairs = sizeof(R) == 4;
-    double s = 0.0;
+    cpx<R> v[E];
     if constexpr (sizeof(R) == 4) {
-        Sum2 kin;
+        const EnergyPre pre = reinterpret_cast<const EnergyPre *>(a.pre)[idx];
+        Pair pot{};
+        if (active) pot = potential_pairs(ip, pre, psi, t, T, E);
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = active ? psi[t + T * e] : cpx<R>{R(0), R(0)};
+        FftPlan<N, E, ALT>::template run<false, R, 1, true>(v, sm, t, tw, 1 + g);
+        Pair kin{};
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            const float m = (float)(t + T * e - (2 * e < E ? 0 : N));
-            add_m2_abs2(kin, m * m, v[e]);
+            const float m = (float)(t + T * e - (2 * e < E ? 0 : N));  // m^2 is exact
+            const Pair d = abs2(v[e]);
+            kin = add(kin, mul(Pair{m * m, 0.0f}, d));
         }
-        s = team_sum<T>((double)kin.hi + (double)kin.lo, slots);
-        // pairs hold 48 bits while squares stay clear of FP32's range; a state of
-        // another size (or not finite) is summed in FP64
-        pairs = !active || (s > 1e-18 && s < 1e30);
+        const double s = team_sum<T>(kin, slots), p = team_sum<T>(pot, slots);
+        // pairs hold 46 bits while squares stay clear of FP32's range: sum |v|^2 >=
+        // 4 s / N^3; a state of another size (or not finite) is summed in FP64
+        bool pairs = !active || (s > 1e-12 * N * N * N && s < 1e30 && p > -1e30 && p < 1e30);
         if constexpr (T < 32) pairs = __all_sync(0xffffffffu, pairs);
+        if (pairs) {
+            if (active && t == 0) a.out[2 * idx + 1] = fma(s, ck, p) * ip.dx[0];
+            return;
+        }
     }
-    if (!pairs) {
-        double kin = 0.0;
+    double pot = 0.0, kin = 0.0;
+    if constexpr (sizeof(R) == 4) {
+        if (active) pot = potential_wide(ip, *a.t_dev, psi, t, T, E);
+        // in a loop through the exchange buffer: its last readers are behind team_sum
+#pragma unroll
+        for (int e = 0; e < E; ++e) sm[t + T * e] = v[e];
+#pragma unroll 1
+        for (int e = 0; e < E; ++e) {
+            const double m = t + T * e - (2 * e < E ? 0 : N), vx = sm[t + T * e].x, vy = sm[t + T * e].y;
+            kin = fma(m * m, fma(vx, vx, vy * vy), kin);
+        }
+    } else {
+        const StageFGE pre = a.pre[idx];
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = active ? psi[t + T * e] : cpx<R>{R(0), R(0)};
+        if (active) pot = potential_fp64<N, E>(ip, v, t, pre.f, pre.g, pre.e);
+        FftPlan<N, E, ALT>::template run<false, R, 1, true>(v, sm, t, tw, 1 + g);
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int m = t + T * e - (2 * e < E ? 0 : N);
-            const double vx = v[e].x, vy = v[e].y;
-            kin = fma(square64(m), fma(vx, vx, vy * vy), kin);
+            kin = fma(square64(m), fma(v[e].x, v[e].x, v[e].y * v[e].y), kin);
         }
-        s = team_sum<T>(kin, slots);
     }
-    s = fma(s, ck, team_sum<T>(pot, slots));
-    if (active && t == 0) a.out[2 * idx + 1] = s * ip.dx[0];
+    kin = team_sum<T>(kin, slots);
+    kin = fma(kin, ck, team_sum<T>(pot, slots));
+    if (active && t == 0) a.out[2 * idx + 1] = kin * ip.dx[0];
 }
 
 // What every thread of an instance needs, once per instance: mu omega^2 / 2 and
 // cos, sin of k T dx (with the law's sine and this sincos in every thread the two
-// calls took 0.34 ms)
-__global__ void energy_pre_kernel(const Diag1DArgs a)
+// calls took 0.34 ms); for an FP32 state in pairs.
+template <typename R> __global__ void energy_pre_kernel(const Diag1DArgs a)
 {
     const int w = blockIdx.x, i = threadIdx.x;
     const WorkItem it = a.work[w];
     if (i >= it.count) return;
     const int idx = a.order[it.first + i];
     const DevInst &ip = a.inst[idx];
-    StageFGE r{};
-    r.f = 0.5 * ip.mu * law_omega2(ip, *a.t_dev);
-    sincos(ip.vi_k * (ip.dx[0] * (ip.n[0] / plan_ept(it.diag))), &r.e, &r.g);
-    a.pre[idx] = r;
+    const double c2 = 0.5 * ip.mu * law_omega2(ip, *a.t_dev);
+    double sn, cs;
+    sincos(ip.vi_k * (ip.dx[0] * (ip.n[0] / plan_ept(it.diag))), &sn, &cs);
+    if constexpr (sizeof(R) == 8) {
+        StageFGE r{};
+        r.f = c2;
+        r.g = cs;
+        r.e = sn;
+        a.pre[idx] = r;
+    } else {
+        const double dx = ip.dx[0], d2 = dx * dx, ca = c2 * d2, cb = ip.eps * d2 * d2, r = ip.xc[0] / dx;
+        const bool cosine = ip.vi_kind_eff == HFS_VI_COS;
+        // zero, or within 1e-12 .. 1e8: with |m + r| <= 1e5 and |psi|^2 <= 1e6 no
+        // product leaves FP32's range and no error term that counts underflows
+        auto fits = [](double c) { return c == 0.0 || (fabs(c) >= 1e-12 && fabs(c) <= 1e8); };
+        const bool ok = fabs(r) <= 9e4 && fits(ca) && fits(0.5 * ip.sigma) && fits(cosine ? ip.eps : cb);
+        EnergyPre p;
+        p.r = to_pair(r);
+        p.a = ok ? to_pair(ca) : Pair{__int_as_float(0x7fffffff), 0.0f};
+        p.b = to_pair(cosine ? cs : cb);
+        p.e = to_pair(sn);
+        reinterpret_cast<EnergyPre *>(a.pre)[idx] = p;
+    }
 }
 
 // items of a batch hold about the same number of points each, so CTAs take them
 // in turn
-template <typename R, bool ENERGY> __global__ void __launch_bounds__(kCtaThreads) diag1d_kernel(const Diag1DArgs a)
+template <typename R, bool ENERGY>
+__global__ void __launch_bounds__(kCtaThreads, sizeof(R) == 8 ? 1 : ENERGY ? 2 : 4) diag1d_kernel(const Diag1DArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cpx<R> *smem = reinterpret_cast<cpx<R> *>(smem_raw);
@@ -265,7 +442,7 @@ template <typename R, bool ENERGY> static cudaError_t diag_t(const Diag1DArgs &a
         if (e != cudaSuccess) return e;
         per_sm = std::max(1, n);
     }
-    if (ENERGY) energy_pre_kernel<<<a.nwork, 64, 0, st>>>(a);  // at most 64 instances an item
+    if (ENERGY) energy_pre_kernel<R><<<a.nwork, 64, 0, st>>>(a);  // at most 64 instances an item
     diag1d_kernel<R, ENERGY><<<std::max(1, std::min(a.nwork, sms * per_sm)), kCtaThreads, bytes, st>>>(a);
     return cudaGetLastError();
 }

@@ -1,5 +1,7 @@
 """Few instances: warps of a CTA without an instance, and the FP64 phases
 (perturbation kinds, off-centre boxes, both splits) against the oracle."""
+import math
+
 import numpy as np
 import pytest
 
@@ -140,6 +142,46 @@ def test_norm_and_energy(precision, scale, vi, shift):
         want = dx * (kin + np.sum((0.5 * w0 ** 2 * x ** 2 + inst.eps * v) * d + 0.5 * inst.sigma * d * d))
         assert abs(norm[i] - dx * d.sum()) <= 1e-12 * dx * d.sum()
         assert abs(energy[i] - want) <= (1e-6 if precision == "c64" else 1e-12) * abs(want), (n, i)
+
+
+@pytest.mark.parametrize("n,ept", [(128, 16), (128, 8), (512, 16), (512, 8), (1024, 16), (1024, 4), (2048, 8), (4096, 16)])
+@pytest.mark.parametrize("vi,shift", [(W.VI_COS, False), (W.VI_COS, True), (W.VI_X4, True), (W.VI_NONE, False)])
+def test_fp32_state_sums_in_pairs(n, ept, vi, shift):
+    """An FP32 state's norm and potential energy are summed in floats with exact
+    products.  Norm: at most 15 FP64 additions of exact partial sums and one
+    product with dx (2^-53 each: 2e-15).  Potential: the difference of the
+    energies of one state under two potentials (their kinetic parts are the same
+    number); pairs round at 2^-46, the cosine recurrence over 16 points adds
+    16^2 of these: 1e-11 of the sum of the terms' magnitudes, and the rounding of
+    the two energies."""
+    need_gpu()
+    from paper_1007_3470_gb300 import hfs
+    one, psis = _instances(n, 5, vi, shift, seed=n + 1)
+    two, _ = _instances(n, 5, vi, shift, seed=n + 1)
+    for inst in two:
+        inst.eps, inst.sigma, inst.w0 = 0.0, 0.0, 0.5 * inst.w0
+    psis = [np.asarray(p).astype(np.complex64) for p in psis]
+    got = []
+    for insts in (one, two):
+        s = hfs.Solver(insts, precision="c64", chunk_steps=4)
+        s.set_plan(n, ept)
+        s.set_psi(psis)
+        got.append((s.norm(), s.energy()))
+        s.close()
+    for i, inst in enumerate(one):
+        u = psis[i].astype(np.complex128)
+        x = inst.x()
+        dx = x[1] - x[0]
+        d = u.real ** 2 + u.imag ** 2
+        v = {W.VI_NONE: 0 * x, W.VI_X4: x ** 4, W.VI_COS: np.cos(inst.vi_k * x)}[vi]
+        trap = [0.5 * (q.w0 * x) ** 2 * (1 + q.law[0] * np.sin(q.law[2])) ** 2 for q in (inst, two[i])]
+        terms = [trap[0], -trap[1], inst.eps * v, 0.5 * inst.sigma * d]
+        want = dx * math.fsum((sum(terms) * d).tolist())
+        size = dx * sum(np.sum(np.abs(t) * d) for t in terms)
+        e0, e1 = got[0][1][i], got[1][1][i]
+        assert abs((e0 - e1) - want) <= 1e-11 * size + 1e-15 * (abs(e0) + abs(e1)), i
+        exact = dx * math.fsum((u.real ** 2).tolist() + (u.imag ** 2).tolist())
+        assert abs(got[0][0][i] - exact) <= 2e-15 * exact, i
 
 
 @pytest.mark.parametrize("n", [256, 512, 1024, 2048, 4096])
