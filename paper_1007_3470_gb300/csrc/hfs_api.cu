@@ -920,6 +920,8 @@ static int run_diag(hfs_ctx_s *c, bool energy)
         a.t_dev = wptr<double>(c, c->lay.tdev);
         a.out = dout;
         a.pre = wptr<StageFGE>(c, c->lay.fge);  // free between calls
+        a.count = c->count;
+        for (const WorkItem &w : c->work) a.ept[w.diag / kPlanCodes] = plan_ept(w.diag);
         CK(launch_diag1d(fp64, energy, a, c->sm_count, c->stream));
     } else {
         Diag3DArgs a{};

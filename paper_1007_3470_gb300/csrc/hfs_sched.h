@@ -107,6 +107,8 @@ struct Diag1DArgs {
     const double *t_dev;
     double *out;    // [count][2]: norm, energy
     StageFGE *pre;  // energy: scratch, one record per instance
+    int64_t count;
+    int32_t ept[kNumSizes];  // values per thread of the diagnostics' plans
 };
 // the energies (energy) or the norms of the batch
 cudaError_t launch_diag1d(bool fp64, bool energy, const Diag1DArgs &a, int sms, cudaStream_t st);

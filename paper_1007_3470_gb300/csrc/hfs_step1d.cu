@@ -99,6 +99,30 @@ template <int T> __device__ __forceinline__ double team_sum(Pair s, double *slot
 // the FP64 pipe bounds it (a complex128 state's still); an FP32 state's squares
 // are summed exactly in three floats (to 2^-72), 44 FP32 instructions a point.
 // Squares outside FP32's range, or not finite, are summed again in FP64.
+// One copy of the loop for all plans: unrolled in each, a warp waited for
+// instructions 8 cycles of the 24 it took per issue (37 us for 4096 instances; 30
+// us now).
+__device__ __noinline__ double norm_floats(const cpx<float> *psi, int T, int E)
+{
+    float hi = 0.0f, mid = 0.0f, lo = 0.0f;
+#pragma unroll 1
+    for (int e0 = 0; e0 < E; e0 += 4) {
+        cpx<float> v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = psi[T * (e0 + e)];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const Pair x = two_prod(v[e].x, v[e].x), y = two_prod(v[e].y, v[e].y);
+            const Pair d = two_sum(x.hi, y.hi), r = two_sum(x.lo, y.lo);
+            const Pair h = two_sum(hi, d.hi);
+            const Pair m0 = two_sum(mid, h.lo), m1 = two_sum(m0.hi, d.lo), m2 = two_sum(m1.hi, r.hi);
+            hi = h.hi;
+            mid = m2.hi;
+            lo += (m0.lo + m1.lo) + (m2.lo + r.lo);
+        }
+    }
+    return (double)hi + ((double)mid + (double)lo);
+}
 template <typename R, int T, int E>
 __device__ __forceinline__ void norm_item(const Diag1DArgs &a, const WorkItem &it, double *slots)
 {
@@ -110,21 +134,7 @@ __device__ __forceinline__ void norm_item(const Diag1DArgs &a, const WorkItem &i
     double s = 0.0;
     bool done = false;
     if constexpr (sizeof(R) == 4) {
-        cpx<R> v[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) v[e] = active ? psi[t + T * e] : cpx<R>{R(0), R(0)};
-        float hi = 0.0f, mid = 0.0f, lo = 0.0f;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const Pair x = two_prod(v[e].x, v[e].x), y = two_prod(v[e].y, v[e].y);
-            const Pair d = two_sum(x.hi, y.hi), r = two_sum(x.lo, y.lo);
-            const Pair h = two_sum(hi, d.hi);
-            const Pair m0 = two_sum(mid, h.lo), m1 = two_sum(m0.hi, d.lo), m2 = two_sum(m1.hi, r.hi);
-            hi = h.hi;
-            mid = m2.hi;
-            lo += (m0.lo + m1.lo) + (m2.lo + r.lo);
-        }
-        s = team_sum<T>((double)hi + ((double)mid + (double)lo), slots);
+        s = team_sum<T>(active ? norm_floats(psi + t, T, E) : 0.0, slots);
         done = !active || (s > 1e-18 && s < 1e30);
         if constexpr (T < 32) done = __all_sync(0xffffffffu, done);
     }
@@ -192,9 +202,9 @@ static_assert(sizeof(EnergyPre) == sizeof(StageFGE), "one record per instance");
 // the first cosines.  One copy of the code for all plans, reading the points from
 // memory: unrolled over registers it spilled, and its fetch cost more than its
 // issue.
-__device__ __noinline__ Pair potential_pairs(const DevInst &ip, const EnergyPre &pre, const cpx<float> *psi, int t, int T, int E)
+__device__ __noinline__ Pair potential_pairs(const DevInst &ip, const EnergyPre &pre, Pair hs, const cpx<float> *psi, int t,
+                                             int T, int E)
 {
-    const Pair hs = to_pair(0.5 * ip.sigma);
     const int kind = ip.vi_kind_eff, n = T * E;
     Pair c{}, cn{};
     if (kind == HFS_VI_COS) {
@@ -253,7 +263,7 @@ __device__ __noinline__ double potential_wide(const DevInst &ip, double now, con
 // Energy.  4096 mixed-size FP32 instances: norm and energy took 1.19 ms together
 // (copies included) as two runs of one kernel with cos and all sums in FP64,
 // 0.32 ms with cos by recurrence and the kinetic sum in pairs, which left the FP64
-// pipe 62 % (energy) and 80 % (norm) busy; 0.19 ms with every sum of an FP32 state
+// pipe 62 % (energy) and 80 % (norm) busy; 0.17 ms with every sum of an FP32 state
 // in floats and two CTAs an SM (128 registers; FP64 sums over registers took 255).
 template <typename R, int N, int E, bool ALT>
 __device__ __forceinline__ void energy_item(const Diag1DArgs &a, const WorkItem &it, cpx<R> *smem, double *slots)
@@ -268,12 +278,11 @@ __device__ __forceinline__ void energy_item(const Diag1DArgs &a, const WorkItem 
     const cpx<R> *psi = reinterpret_cast<const cpx<R> *>(a.psi) + ip.off;
     cpx<R> *sm = smem + g * smem_elems(N);
     const auto *tw = reinterpret_cast<const typename TwOf<R>::type *>(a.tw);
-    const double ku = 2.0 * 3.14159265358979323846 / ip.len[0], ck = ku * ku / N / (2.0 * ip.mu);
     cpx<R> v[E];
     if constexpr (sizeof(R) == 4) {
         const EnergyPre pre = reinterpret_cast<const EnergyPre *>(a.pre)[idx];
         Pair pot{};
-        if (active) pot = potential_pairs(ip, pre, psi, t, T, E);
+        if (active) pot = potential_pairs(ip, pre, reinterpret_cast<const Pair *>(a.out)[2 * idx], psi, t, T, E);
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = active ? psi[t + T * e] : cpx<R>{R(0), R(0)};
         FftPlan<N, E, ALT>::template run<false, R, 1, true>(v, sm, t, tw, 1 + g);
@@ -290,7 +299,7 @@ __device__ __forceinline__ void energy_item(const Diag1DArgs &a, const WorkItem 
         bool pairs = !active || (s > 1e-12 * N * N * N && s < 1e30 && p > -1e30 && p < 1e30);
         if constexpr (T < 32) pairs = __all_sync(0xffffffffu, pairs);
         if (pairs) {
-            if (active && t == 0) a.out[2 * idx + 1] = fma(s, ck, p) * ip.dx[0];
+            if (active && t == 0) a.out[2 * idx + 1] = fma(s, a.out[2 * idx + 1], p) * ip.dx[0];
             return;
         }
     }
@@ -318,23 +327,27 @@ __device__ __forceinline__ void energy_item(const Diag1DArgs &a, const WorkItem 
         }
     }
     kin = team_sum<T>(kin, slots);
-    kin = fma(kin, ck, team_sum<T>(pot, slots));
-    if (active && t == 0) a.out[2 * idx + 1] = kin * ip.dx[0];
+    pot = team_sum<T>(pot, slots);
+    if (active && t == 0) a.out[2 * idx + 1] = fma(kin, a.out[2 * idx + 1], pot) * ip.dx[0];
 }
 
 // What every thread of an instance needs, once per instance: mu omega^2 / 2 and
 // cos, sin of k T dx (with the law's sine and this sincos in every thread the two
 // calls took 0.34 ms); for an FP32 state in pairs.
+// One thread per instance (a CTA per work item left most lanes idle: 16 us for
+// 4096 instances, 11 us now, the latency of one thread).  The energy's slots of out hold the kinetic factor and, for an
+// FP32 state, sigma / 2 until the energy is written.
 template <typename R> __global__ void energy_pre_kernel(const Diag1DArgs a)
 {
-    const int w = blockIdx.x, i = threadIdx.x;
-    const WorkItem it = a.work[w];
-    if (i >= it.count) return;
-    const int idx = a.order[it.first + i];
+    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (idx >= a.count) return;
     const DevInst &ip = a.inst[idx];
+    const int n = ip.n[0];
+    const double ku = 2.0 * 3.14159265358979323846 / ip.len[0];
+    a.out[2 * idx + 1] = ku * ku / n / (2.0 * ip.mu);
     const double c2 = 0.5 * ip.mu * law_omega2(ip, *a.t_dev);
     double sn, cs;
-    sincos(ip.vi_k * (ip.dx[0] * (ip.n[0] / plan_ept(it.diag))), &sn, &cs);
+    sincos(ip.vi_k * (ip.dx[0] * (n / a.ept[size_class(n)])), &sn, &cs);
     if constexpr (sizeof(R) == 8) {
         StageFGE r{};
         r.f = c2;
@@ -354,6 +367,7 @@ template <typename R> __global__ void energy_pre_kernel(const Diag1DArgs a)
         p.b = to_pair(cosine ? cs : cb);
         p.e = to_pair(sn);
         reinterpret_cast<EnergyPre *>(a.pre)[idx] = p;
+        reinterpret_cast<Pair *>(a.out)[2 * idx] = to_pair(0.5 * ip.sigma);
     }
 }
 
@@ -442,7 +456,7 @@ template <typename R, bool ENERGY> static cudaError_t diag_t(const Diag1DArgs &a
         if (e != cudaSuccess) return e;
         per_sm = std::max(1, n);
     }
-    if (ENERGY) energy_pre_kernel<R><<<a.nwork, 64, 0, st>>>(a);  // at most 64 instances an item
+    if (ENERGY) energy_pre_kernel<R><<<(unsigned)((a.count + 63) / 64), 64, 0, st>>>(a);
     diag1d_kernel<R, ENERGY><<<std::max(1, std::min(a.nwork, sms * per_sm)), kCtaThreads, bytes, st>>>(a);
     return cudaGetLastError();
 }
