@@ -83,7 +83,10 @@ int hfs_fno_train_step(hfs_fno_t f, const float *x_dev, const float *y_dev, int3
 
 /* GEMM engine of the row-streaming products (rows >= 8192, K and N of 64 or
  * 128: the pointwise layers, the projection and their backward products).
- * HFS_FNO_GEMM_MMA_SYNC (default): cp.async tile ring and mma.sync.m16n8k16.
+ * HFS_FNO_GEMM_MMA_SYNC (default): for width 16, 32 or 64, power-of-two grids
+ * 32..256, modes 8..64 and proj 16..256 (training: up to 128; all powers of
+ * two) and out_ch <= 8 the fused per-sample passes, otherwise GEMM by GEMM
+ * with a cp.async tile ring; mma.sync.m16n8k16 in both.
  * HFS_FNO_GEMM_TCGEN05: persistent CTAs keep op(B) in shared memory, stream
  * 128-row tiles of A, and run the products on the tcgen05 tensor cores (BF16
  * operands through shared-memory descriptors, FP32 accumulators in tensor

@@ -331,12 +331,12 @@ __device__ __forceinline__ void energy_item(const Diag1DArgs &a, const WorkItem 
     if (active && t == 0) a.out[2 * idx + 1] = fma(kin, a.out[2 * idx + 1], pot) * ip.dx[0];
 }
 
-// What every thread of an instance needs, once per instance: mu omega^2 / 2 and
-// cos, sin of k T dx (with the law's sine and this sincos in every thread the two
-// calls took 0.34 ms); for an FP32 state in pairs.
-// One thread per instance (a CTA per work item left most lanes idle: 16 us for
-// 4096 instances, 11 us now, the latency of one thread).  The energy's slots of out hold the kinetic factor and, for an
-// FP32 state, sigma / 2 until the energy is written.
+// What every thread of an instance needs, once per instance: mu omega^2 / 2, cos,
+// sin of k T dx and the kinetic factor (with the law's sine and this sincos in
+// every thread the two calls took 0.34 ms); for an FP32 state in pairs.  One
+// thread per instance: a CTA per work item left most lanes idle (16 us for 4096
+// instances, 11 us now, the latency of one thread).  The energy's slots of out
+// hold the kinetic factor and, for an FP32 state, sigma / 2 until it is written.
 template <typename R> __global__ void energy_pre_kernel(const Diag1DArgs a)
 {
     const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
