@@ -240,31 +240,40 @@ __device__ __forceinline__ void apply_turns2(cpx<float> &u0, cpx<float> &u1, flo
 // FP64 pipe is the bound of every FP64 kernel here (2 lanes a cycle on an SM),
 // so its instructions are counted: the quarter turn is split off in three (the
 // additions of 1.5 2^52 round to nearest as kRoundMagic does), and sin and cos
-// of the rest |f| <= 1/8 turn take sixteen, near-minimax polynomials in f^2
-// (Remez, errors 3.4e-18 relative and 3.3e-20) with 2 pi and the scale in their
-// coefficients; the quarter turn itself is swaps and signs on the integer
-// pipe.  sincospi on the reduced phase took 35.  With cos(k x) from a table as
-// well, 700 FP64 instances of 2048 points: 3.23 -> 2.30 ms per 5 steps.
+// of the rest |f| <= 1/8 turn take sixteen, sin 2 pi f = f (2 pi + f^2 Q) with 2 pi
+// as an unevaluated sum and cos 2 pi f = 1 + f^2 P, the scale in the coefficients.
+// P and Q are minimax polynomials in f^2 (Remez), the coefficients rounded to FP64
+// one at a time with the later ones refitted (fit_rotation_poly.py): errors 4.2e-18
+// relative (sin) and 1.3e-18 (cos) before the evaluation's own roundings.  (With 2 pi
+// rounded, 3.9e-17 relative, complex128 runs ended 1 to 2.5 % further off.)  The
+// quarter turn itself is swaps and signs on the integer pipe.  sincospi on the
+// reduced phase took 35.  With cos(k x) from a table as well, 700 FP64 instances of
+// 2048 points: 3.23 -> 2.30 ms per 5 steps.
 constexpr double kRoundMagic64 = 6755399441055744.0;  // 1.5 * 2^52
+constexpr double kTwoPi64 = 6.283185307179586, kTwoPi64Lo = 2.4492935982947064e-16;
+constexpr double kSinF3 = -41.34170224039967, kSinF5 = 81.60524927596379, kSinF7 = -76.70585970743427,
+                 kSinF9 = 42.05868532107631, kSinF11 = -15.093817508161722, kSinF13 = 3.7810851140590542;
+constexpr double kCosF2 = -19.739208802178716, kCosF4 = 64.93939402266663, kCosF6 = -85.45681720595688,
+                 kCosF8 = 60.24464121866748, kCosF10 = -26.426240104378916, kCosF12 = 7.902573801368685,
+                 kCosF14 = -1.6872164068523487;
 __device__ __forceinline__ cpx<double> apply_turns(cpx<double> u, double turns, double scale)
 {
     const double tq = fma(4.0, turns, kRoundMagic64);
     const double f = fma(tq - kRoundMagic64, -0.25, turns);
     const double f2 = f * f;
-    double ps = fma(f2, 0.6018231468337394, -2.4022575464993303);
-    ps = fma(ps, f2, 6.693847698340711);
-    ps = fma(ps, f2, -12.208116736766483);
-    ps = fma(ps, f2, 12.987878804516656);
-    ps = fma(ps, f2, -6.579736267392892);
-    const double th = f * (6.28318530717958647692 * scale);
-    const double s = fma(th * f2, ps, th);
-    double pc = fma(f2, -1.6970200893650267 * scale, 7.903101638520154 * scale);
-    pc = fma(pc, f2, -26.426251140438435 * scale);
-    pc = fma(pc, f2, 60.2446413316117 * scale);
-    pc = fma(pc, f2, -85.45681720654005 * scale);
-    pc = fma(pc, f2, 64.93939402266801 * scale);
-    pc = fma(pc, f2, -19.739208802178716 * scale);
-    const double c = fma(f2, pc, scale);
+    double ps = fma(f2, kSinF13 * scale, kSinF11 * scale);
+    ps = fma(ps, f2, kSinF9 * scale);
+    ps = fma(ps, f2, kSinF7 * scale);
+    ps = fma(ps, f2, kSinF5 * scale);
+    ps = fma(ps, f2, kSinF3 * scale);
+    ps = fma(ps, f2, kTwoPi64Lo * scale);
+    double pc = fma(f2, kCosF14 * scale, kCosF12 * scale);
+    pc = fma(pc, f2, kCosF10 * scale);
+    pc = fma(pc, f2, kCosF8 * scale);
+    pc = fma(pc, f2, kCosF6 * scale);
+    pc = fma(pc, f2, kCosF4 * scale);
+    pc = fma(pc, f2, kCosF2 * scale);
+    const double s = fma(f, ps, f * (kTwoPi64 * scale)), c = fma(f2, pc, scale);
     const double wx = fma(u.x, c, u.y * s), wy = fma(u.y, c, -(u.x * s));
     // (-i)^q: as finish_rotation
     const int q = __double2loint(tq) & 3;

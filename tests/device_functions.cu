@@ -1,0 +1,36 @@
+// Device functions of the library over their whole ranges, one check a call; built
+// and run by test_gpu_device_functions.py.
+#include <cstdio>
+#include <cstring>
+
+#include "hfs_phase.cuh"
+
+using namespace hfs;
+
+__device__ void atomic_max(double *p, double v)  // of values >= 0
+{
+    atomicMax(reinterpret_cast<unsigned long long *>(p), (unsigned long long)__double_as_longlong(v));
+}
+
+// apply_turns in FP64 against sincospi: turns over 2^-60 .. 2^40 (uniform in the
+// exponent) of either sign
+__global__ void turns_error(double *worst)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, n = gridDim.x * blockDim.x;
+    const double turns = (i & 1 ? -1.0 : 1.0) * exp2(-60.0 + 100.0 * i / n);
+    const cpx<double> v = apply_turns(cpx<double>{1.0, 0.0}, turns, 1.0);
+    double s, c;
+    sincospi(2.0 * (turns - rint(turns)), &s, &c);
+    atomic_max(worst, fmax(fabs(v.x - c), fabs(v.y + s)));
+}
+
+int main(int, char **argv)
+{
+    double *d = nullptr, h = 0.0;
+    if (cudaMalloc(&d, 8) != cudaSuccess || cudaMemset(d, 0, 8) != cudaSuccess) return 1;
+    if (!strcmp(argv[1], "turns_error")) turns_error<<<4096, 256>>>(d);
+    else return 1;
+    if (cudaMemcpy(&h, d, 8, cudaMemcpyDeviceToHost) != cudaSuccess) return 1;
+    printf("%.17g\n", h);
+    return cudaFree(d) != cudaSuccess;
+}
