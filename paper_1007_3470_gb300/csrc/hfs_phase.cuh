@@ -248,7 +248,11 @@ __device__ __forceinline__ void apply_turns2(cpx<float> &u0, cpx<float> &u1, flo
 // rounded, 3.9e-17 relative, complex128 runs ended 1 to 2.5 % further off.)  The
 // quarter turn itself is swaps and signs on the integer pipe.  sincospi on the
 // reduced phase took 35.  With cos(k x) from a table as well, 700 FP64 instances of
-// 2048 points: 3.23 -> 2.30 ms per 5 steps.
+// 2048 points: 3.23 -> 2.30 ms per 5 steps.  At 2^49 turns and more (4 turns
+// + 1.5 2^52 beyond 2^53) the phase has lost its angle and f its bound: the rotation
+// is then a multiple of a quarter turn, of modulus 1 as every other, by selections on
+// the integer pipe (1 % of a step; turns - rint(turns) instead took 5 %).  Not
+// finite turns give NaN.
 constexpr double kRoundMagic64 = 6755399441055744.0;  // 1.5 * 2^52
 constexpr double kTwoPi64 = 6.283185307179586, kTwoPi64Lo = 2.4492935982947064e-16;
 constexpr double kSinF3 = -41.34170224039967, kSinF5 = 81.60524927596379, kSinF7 = -76.70585970743427,
@@ -273,7 +277,9 @@ __device__ __forceinline__ cpx<double> apply_turns(cpx<double> u, double turns, 
     pc = fma(pc, f2, kCosF6 * scale);
     pc = fma(pc, f2, kCosF4 * scale);
     pc = fma(pc, f2, kCosF2 * scale);
-    const double s = fma(f, ps, f * (kTwoPi64 * scale)), c = fma(f2, pc, scale);
+    // 2^49 <= |turns| < infinity
+    const bool far = (unsigned)((__double2hiint(turns) & 0x7fffffff) - 0x43000000) < 0x7ff00000u - 0x43000000u;
+    const double s = far ? 0.0 : fma(f, ps, f * (kTwoPi64 * scale)), c = far ? scale : fma(f2, pc, scale);
     const double wx = fma(u.x, c, u.y * s), wy = fma(u.y, c, -(u.x * s));
     // (-i)^q: as finish_rotation
     const int q = __double2loint(tq) & 3;

@@ -24,11 +24,22 @@ __global__ void turns_error(double *worst)
     atomic_max(worst, fmax(fabs(v.x - c), fabs(v.y + s)));
 }
 
+// its modulus over all finite turns
+__global__ void turns_modulus(double *worst)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, n = gridDim.x * blockDim.x;
+    const double turns = (i & 1 ? -1.0 : 1.0) * exp2(-1000.0 + 2023.9 * i / n);
+    const cpx<double> v = apply_turns(cpx<double>{0.8, -0.6}, turns, 1.0);
+    const double e = fabs(v.x * v.x + v.y * v.y - 1.0);
+    atomic_max(worst, e >= 0.0 ? e : 1e300);
+}
+
 int main(int, char **argv)
 {
     double *d = nullptr, h = 0.0;
     if (cudaMalloc(&d, 8) != cudaSuccess || cudaMemset(d, 0, 8) != cudaSuccess) return 1;
     if (!strcmp(argv[1], "turns_error")) turns_error<<<4096, 256>>>(d);
+    else if (!strcmp(argv[1], "turns_modulus")) turns_modulus<<<4096, 256>>>(d);
     else return 1;
     if (cudaMemcpy(&h, d, 8, cudaMemcpyDeviceToHost) != cudaSuccess) return 1;
     printf("%.17g\n", h);
