@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane3d(const Step3DArgs a, 
 // transform each at a time) and every launch programmatic.  Bound by latency:
 // the state lies in L2 and a pass is one chain of load, transforms and store.
 // Four line passes took 17.8 us a step at 64^3 and 17.8 us at 32^3 (27 us without
-// graph replay); these take 8.3 us and 6.1 us (6.9 us).
+// graph replay); these take 8.4 us and 4.3 us.
 // ---------------------------------------------------------------------------
 template <int N> struct Cube {
     static constexpr int E = 8, T = N / E, ROW = smem_elems(N);
