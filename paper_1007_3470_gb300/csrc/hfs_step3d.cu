@@ -40,9 +40,9 @@ template <int N> struct Geo3 {
 // the smaller grids are cut into CTAs of one or two warps (64^3 as 64 CTAs of 256
 // threads left more than half of the SMs idle: 196 us a step of phases and
 // transforms, 107 us now; 32^3 125 us, 48 us now).
-template <typename R, int N, bool PROJ = false> struct LineGeo {
+template <typename R, int N> struct LineGeo {
     static constexpr bool kSmall = sizeof(R) == 8 && N < 128;
-    static constexpr int E = kSmall || PROJ ? 8 : 16, T = N / E;
+    static constexpr int E = kSmall ? 8 : 16, T = N / E;
     static constexpr int THREADS = !kSmall ? kCtaThreads : N == 32 ? 32 : 64;
     static constexpr int G = THREADS / T;
     static constexpr int TX = G < N ? G : N;
@@ -151,14 +151,12 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // z-pass: one CTA = fixed y, TX adjacent x columns; forward FFT_z, k-phase,
 // inverse FFT_z
 // ---------------------------------------------------------------------------
-// FP32 with the norm projection (plain twiddles): eight values a thread and four
-// CTAs per SM of 64 registers, twice the warps behind the column loads (100
-// steps at 128^3: 2.99 -> 2.92 ms).  Without it the third pass's compensated
-// twiddles cost more than that (20 steps 0.68 against 0.65 ms): sixteen values and
-// two CTAs of 128 registers.  FP64: one CTA
-template <typename R, bool PROJ> struct ZpassMinCtas {
-    static constexpr int value = sizeof(R) == 4 ? (PROJ ? 4 : 2) : 1;
-};
+// FP32: two CTAs per SM (128 registers; at 143 registers one CTA of 8 warps
+// per SM left the column loads' latency exposed); FP64: one.  Eight values a thread
+// and four CTAs of 64 registers took 2.92 instead of 2.99 ms for 100 projected steps
+// of 128^3, but a third pass under plain twiddles left the state 5.5 % further from
+// 64 bits (60 steps: 1.745e-6 -> 1.841e-6).
+template <typename R> struct ZpassMinCtas { static constexpr int value = sizeof(R) == 4 ? 2 : 1; };
 // Norm projection in 3D: the plane pass of sub-stage j adds its plane's sum
 // of |u|^2 (taken in the x-phase) to slot j mod 3; the z-pass j that follows
 // reads the complete sum, scales its k-phase by C = sqrt(target / sum), and
@@ -196,11 +194,10 @@ __device__ __forceinline__ void fft3(cpx<R> (&v)[E], cpx<R> *sm, int t, const St
 }
 
 template <typename R, int N, bool PROJ = false>
-__global__ void __launch_bounds__(LineGeo<R, N>::THREADS, ZpassMinCtas<R, PROJ>::value)
-    zpass3d(const Step3DArgs a, int64_t j)
+__global__ void __launch_bounds__(LineGeo<R, N>::THREADS, ZpassMinCtas<R>::value) zpass3d(const Step3DArgs a, int64_t j)
 {
     using Rec = typename Rec3Of<R>::type;
-    using GEO = LineGeo<R, N, PROJ>;
+    using GEO = LineGeo<R, N>;
     constexpr int E = GEO::E, T = GEO::T, TX = GEO::TX;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int l = threadIdx.x % TX, t = threadIdx.x / TX;
@@ -819,7 +816,7 @@ template <int N> static cudaError_t run3d_cube(const Step3DArgs &a, cudaStream_t
 template <int VI, bool PROJ> static cudaError_t run3d_plane_vi(const Step3DArgs &a, cudaStream_t st)
 {
     constexpr int N = kPlaneN;
-    using GEO = LineGeo<float, N, PROJ>;
+    using GEO = LineGeo<float, N>;
     constexpr int FIRST = P_PHASE | P_FWD_X | P_FWD_Y, MID = P_INV_Y | P_INV_X | P_PHASE | P_FWD_X | P_FWD_Y,
                   LAST = P_INV_Y | P_INV_X | P_PHASE;
     const size_t ps = (size_t)N * kPlaneRow * sizeof(cpx<float>), ts = (size_t)GEO::TX * N * sizeof(cpx<float>);
@@ -839,7 +836,7 @@ template <int VI, bool PROJ> static cudaError_t run3d_plane_vi(const Step3DArgs 
     plane3d<FIRST, VI, PROJ><<<N, kPlaneThreads, ps, st>>>(a, 0);
     cudaError_t e = cudaGetLastError();
     for (int64_t j = 0; j < a.nstage && e == cudaSuccess; ++j) {
-        if (a.dft_tc) e = launch_pdl(zpass3d_tc<N, PROJ>, dim3(N / Geo3<N>::TX, N), dim3(Geo3<N>::TT), zpass_tc_smem<N>(), st, a, j);
+        if (a.dft_tc) e = launch_pdl(zpass3d_tc<N, PROJ>, tg, dim3(GEO::TT), zpass_tc_smem<N>(), st, a, j);
         else e = launch_pdl(zpass3d<float, N, PROJ>, tg, dim3(GEO::TT), ts, st, a, j);
         if (e != cudaSuccess) break;
         if (j + 1 < a.nstage) e = launch_pdl(plane3d<MID, VI, PROJ>, dim3(N), dim3(kPlaneThreads), ps, st, a, j + 1);
