@@ -346,12 +346,12 @@ __device__ __forceinline__ void fft_passes(cpx<R> (&v)[E], cpx<R> *sm, int t,
 // radices 4 and 2 on one lane.  The operations on every value are those of
 // stockham_pass, in the same order, so the results are the same bits.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ cpx<float> shfl_xor(cpx<float> a, int m)
+template <typename R> __device__ __forceinline__ cpx<R> shfl_xor(cpx<R> a, int m)
 {
     return {__shfl_xor_sync(0xffffffffu, a.x, m), __shfl_xor_sync(0xffffffffu, a.y, m)};
 }
-// v[j] of lane k <-> v[k] of lane j, for four adjacent lanes
-__device__ __forceinline__ void lane_transpose4(cpx<float> (&v)[4], int q)
+// v[j] of lane k <-> v[k] of lane j, for four lanes LS apart
+template <int LS = 1, typename R> __device__ __forceinline__ void lane_transpose4(cpx<R> (&v)[4], int q)
 {
 #pragma unroll
     for (int m = 1; m <= 2; m <<= 1) {
@@ -359,7 +359,7 @@ __device__ __forceinline__ void lane_transpose4(cpx<float> (&v)[4], int q)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             if (i & m) continue;
-            const cpx<float> r = shfl_xor(hi ? v[i] : v[i | m], m);
+            const cpx<R> r = shfl_xor(hi ? v[i] : v[i | m], m * LS);
             if (hi) v[i] = r;
             else v[i | m] = r;
         }
@@ -402,17 +402,31 @@ template <int K, bool INV> __device__ __forceinline__ cpx<float> lane_rot16(cpx<
         return (q & 1) ? m : even;
     }
 }
-template <bool INV> __device__ __forceinline__ void lane_dft16(cpx<float> (&v)[4], int q)
+// FP64: one product with the lane's constant for every exponent (0 and 4 exact);
+// the FP64 pipe takes 16 cycles a warp instruction, a selection one or two
+template <int K, bool INV> __device__ __forceinline__ cpx<double> lane_rot16(cpx<double> a, int q)
+{
+    static_assert(K >= 1 && K <= 3, "inner transform's outputs");
+    constexpr double C1 = RotConst<double>::c1, S1 = RotConst<double>::s1, R2 = RotConst<double>::r2;
+    // exponents q K: 0 1 2 3, 0 2 4 6, 0 3 6 9
+    constexpr double c1 = K == 1 ? C1 : K == 2 ? R2 : S1, s1 = K == 1 ? -S1 : K == 2 ? -R2 : -C1;
+    constexpr double c2 = K == 1 ? R2 : K == 2 ? 0.0 : -R2, s2 = K == 1 ? -R2 : K == 2 ? -1.0 : -R2;
+    constexpr double c3 = K == 1 ? S1 : K == 2 ? -R2 : -C1, s3 = K == 1 ? -C1 : K == 2 ? -R2 : S1;
+    const double c = (q & 2) ? ((q & 1) ? c3 : c2) : ((q & 1) ? c1 : 1.0);
+    const double s = (q & 2) ? ((q & 1) ? s3 : s2) : ((q & 1) ? s1 : 0.0);
+    return mulw(a, c, INV ? -s : s);
+}
+template <bool INV, int LS = 1, typename R> __device__ __forceinline__ void lane_dft16(cpx<R> (&v)[4], int q)
 {
     dft4s<INV, HFS_PACK_DFT16 != 0>(v[0], v[1], v[2], v[3]);
     v[1] = lane_rot16<1, INV>(v[1], q);
     v[2] = lane_rot16<2, INV>(v[2], q);
     v[3] = lane_rot16<3, INV>(v[3], q);
-    lane_transpose4(v, q);
+    lane_transpose4<LS>(v, q);
     dft4s<INV, HFS_PACK_DFT16 != 0>(v[0], v[1], v[2], v[3]);
 }
 // radix 8 on lanes q (q & 2 == 0: even inputs) and q ^ 2 (odd inputs)
-template <bool INV> __device__ __forceinline__ void lane_dft8(cpx<float> (&v)[4], int q)
+template <bool INV, typename R> __device__ __forceinline__ void lane_dft8(cpx<R> (&v)[4], int q)
 {
     const bool odd = q & 2;
     dft4s<INV, HFS_PACK_DFT8 != 0>(v[0], v[1], v[2], v[3]);
@@ -423,8 +437,8 @@ template <bool INV> __device__ __forceinline__ void lane_dft8(cpx<float> (&v)[4]
     }
     __syncwarp();
     // the even lane forms outputs 0, 2, 4, 6, the odd one 1, 3, 5, 7
-    const cpx<float> r0 = shfl_xor(odd ? v[0] : v[1], 2), r1 = shfl_xor(odd ? v[2] : v[3], 2);
-    const cpx<float> e0 = odd ? r0 : v[0], e1 = odd ? r1 : v[2], o0 = odd ? v[1] : r0, o1 = odd ? v[3] : r1;
+    const cpx<R> r0 = shfl_xor(odd ? v[0] : v[1], 2), r1 = shfl_xor(odd ? v[2] : v[3], 2);
+    const cpx<R> e0 = odd ? r0 : v[0], e1 = odd ? r1 : v[2], o0 = odd ? v[1] : r0, o1 = odd ? v[3] : r1;
     v[0] = cadd(e0, o0);
     v[1] = cadd(e1, o1);
     v[2] = csub(e0, o0);
@@ -473,6 +487,27 @@ template <int N, bool INV> __device__ __forceinline__ void lane_fft(cpx<float> (
     else lane_pass<N, 16, 16, INV, N == 256>(v, sm, b, q, tw);
     if constexpr (N > 256) lane_pass<N, N / 256, 256, INV, true>(v, sm, b, q, tw);
     static_assert(N <= 1024, "radix sequence");
+}
+
+// 32 points of a line on eight threads, four values each (t + 8 e), in one warp: the
+// plan of sixteen values a thread, butterfly b of its first pass on the threads t = b +
+// 2 q; consecutive threads ILV lanes apart, as stockham_pass interleaves lines.
+template <bool INV, int ILV>
+__device__ __forceinline__ void lane_fft32(cpx<double> (&v)[4], cpx<double> *sm, int t, const double2 *tw)
+{
+    const int b = t & 1, q = t >> 1;
+    lane_dft16<INV, 2 * ILV>(v, q);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) sm[sbase<ILV>(b * 16 + q) + soff<ILV>(4 * k)] = v[k];
+    __syncwarp();
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        v[e] = sm[sbase<ILV>(t) + soff<ILV>(8 * e)];
+        if (e >= 2) v[e] = tw_mul<INV>(v[e], tw, (int)tw_pass_offset(32, 2) + t + 8 * (e & 1));
+    }
+    __syncwarp();
+    dft2<INV>(v[0], v[2]);
+    dft2<INV>(v[1], v[3]);
 }
 
 // Radix sequences per (N, elements per thread, ALT: the alternative order).

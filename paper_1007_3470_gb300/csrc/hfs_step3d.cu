@@ -39,15 +39,24 @@ template <int N> struct Geo3 {
 // The line passes.  FP64 is bound by the FP64 pipe of the SMs that hold a CTA, so
 // the smaller grids are cut into CTAs of one or two warps (64^3 as 64 CTAs of 256
 // threads left more than half of the SMs idle: 196 us a step of phases and
-// transforms, 107 us now; 32^3 125 us, 48 us now).
+// transforms, 107 us now).  32^3: four values a thread with the butterflies of
+// sixteen spread over lanes, 125 us, 33 us now (eight values, 8 4: 48 us, and states
+// 20 % further from 64 bits: 4.0e-15 -> 4.8e-15 after 20 steps).
 template <typename R, int N> struct LineGeo {
     static constexpr bool kSmall = sizeof(R) == 8 && N < 128;
-    static constexpr int E = kSmall ? 8 : 16, T = N / E;
+    static constexpr int E = !kSmall ? 16 : N == 32 ? 4 : 8, T = N / E;
     static constexpr int THREADS = !kSmall ? kCtaThreads : N == 32 ? 32 : 64;
     static constexpr int G = THREADS / T;
     static constexpr int TX = G < N ? G : N;
     static constexpr int TT = T * TX;
 };
+
+template <int N, bool INV, int ILV, typename R, int E>
+__device__ __forceinline__ void line_fft(cpx<R> (&v)[E], cpx<R> *sm, int t, const typename TwOf<R>::type *tw)
+{
+    if constexpr (E == 4) lane_fft32<INV, ILV>(v, sm, t, tw);
+    else FftPlan<N, E>::template run<INV, R, ILV>(v, sm, t, tw);
+}
 
 __device__ __forceinline__ float turns_q(int m, float hi, float lo) { return frac_turns((float)(m * m), hi, lo); }
 __device__ __forceinline__ double turns_q(int m, double c, double) { return frac_turns((double)m * m, c, 0.0); }
@@ -83,7 +92,7 @@ __global__ void __launch_bounds__(LineGeo<R, N>::THREADS) xpass3d(const Step3DAr
     cpx<R> v[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = psi[t + T * e];
-    if constexpr (MODE & X_INV) FftPlan<N, E>::template run<true, R>(v, sm, t, tw);
+    if constexpr (MODE & X_INV) line_fft<N, true, 1>(v, sm, t, tw);
     if constexpr (MODE & X_PHASE) {
         const Rec rc = reinterpret_cast<const Rec *>(a.rec)[j];
         const DevInst &ip = *a.inst;
@@ -105,7 +114,7 @@ __global__ void __launch_bounds__(LineGeo<R, N>::THREADS) xpass3d(const Step3DAr
             v[e] = apply_turns(v[e], turns, R(1));
         }
     }
-    if constexpr (MODE & X_FWD) FftPlan<N, E>::template run<false, R>(v, sm, t, tw);
+    if constexpr (MODE & X_FWD) line_fft<N, false, 1>(v, sm, t, tw);
     bool bad = false;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
@@ -132,7 +141,7 @@ __global__ void __launch_bounds__(LineGeo<R, N>::THREADS) ypass3d(const Step3DAr
     cpx<R> v[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = psi[(int64_t)(t + T * e) * N];
-    FftPlan<N, E>::template run<INV, R, TX>(v, sm, t, tw);
+    line_fft<N, INV, TX>(v, sm, t, tw);
 #pragma unroll
     for (int e = 0; e < E; ++e) psi[(int64_t)(t + T * e) * N] = v[e];
 }
@@ -189,8 +198,7 @@ __device__ __forceinline__ void fft3(cpx<R> (&v)[E], cpx<R> *sm, int t, const St
     if constexpr (PROJ && sizeof(R) == 4)
         FftPlan<N, E>::template run<INV, R, ILV, false, false>(v, sm, t, static_cast<const float2 *>(a.tw2));
     else
-        FftPlan<N, E>::template run<INV, R, ILV>(v, sm, t,
-                                                 reinterpret_cast<const typename TwOf<R>::type *>(a.tw));
+        line_fft<N, INV, ILV>(v, sm, t, reinterpret_cast<const typename TwOf<R>::type *>(a.tw));
 }
 
 template <typename R, int N, bool PROJ = false>

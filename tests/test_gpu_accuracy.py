@@ -48,9 +48,11 @@ def test_fp32_radix_8(n):
 # 1.3256e-6) with the 0.6 % that 8 8 is off it, and the 1.354e-6 of sums times
 # sqrt(1/2); 16 seeds have a standard deviation of 2.6e-9.  128^3: midway between
 # sixteen values a thread in the z-pass (1.745e-6) and eight (1.841e-6); 3 seeds 7e-9.
+# 32^3: between 4.0e-15 and the 4.8e-15 of 8 4; 16 seeds 1.5e-16, the same in both.
 @pytest.mark.parametrize("case,seeds,bound", [(_cube(64), 16, 1.3437e-6),
-                                              (_cube(128, steps=60, projection=True), 3, 1.793e-6)],
-                         ids=["64^3 c64", "128^3 c64 projected"])
+                                              (_cube(128, steps=60, projection=True), 3, 1.793e-6),
+                                              (_cube(32, steps=20, precision="c128"), 16, 4.4e-15)],
+                         ids=["64^3 c64", "128^3 c64 projected", "32^3 c128"])
 def test_3d_error(case, seeds, bound):
     need_gpu()
     assert _error(case, range(100, 100 + seeds)) <= bound
