@@ -344,7 +344,8 @@ __device__ __forceinline__ void fft_passes(cpx<R> (&v)[E], cpx<R> *sm, int t,
 // inputs q + 4 e), the twiddles W_16^{q k} depend on the lane, a 4 x 4 transpose
 // by shuffles feeds the outer ones.  A closing radix 8 lies on lanes q and q ^ 2,
 // radices 4 and 2 on one lane.  The operations on every value are those of
-// stockham_pass, in the same order, so the results are the same bits.
+// stockham_pass, in the same order, so that FP32 results are the same bits (FP64: the
+// same radices and factors; the compiler fuses other products into additions there).
 // ---------------------------------------------------------------------------
 template <typename R> __device__ __forceinline__ cpx<R> shfl_xor(cpx<R> a, int m)
 {
@@ -543,10 +544,6 @@ HFS_PLAN(1024, 4, 4, 4, 4, 4, 4)
 HFS_PLAN(512, 4, 4, 4, 4, 4, 2)
 HFS_PLAN(256, 4, 4, 4, 4, 4)
 HFS_PLAN(128, 4, 4, 4, 4, 2)
-// the factors of a transform spread over a cluster (hfs_step1d_cluster.cu)
-HFS_PLAN(64, 4, 4, 4, 4)
-HFS_PLAN(32, 4, 4, 4, 2)
-HFS_PLAN(16, 4, 4, 4)
 // sixteen values per thread, alternative radix orders
 HFS_PLAN_ORDER(4096, 16, true, 8, 8, 8, 8)
 HFS_PLAN_ORDER(2048, 16, true, 8, 16, 16)
