@@ -113,7 +113,7 @@ double omega_bound(const hfs_instance &p, double t0, double t1)
 namespace {
 
 struct Layout {
-    size_t status, ticket, tdev, inst, order, work, twf, twd, twp, fge, nodes, rec, diag, norm, nsum3, rec2, total;
+    size_t status, ticket, tdev, inst, order, work[2], twf, twd, twp, fge, nodes, rec, diag, norm, nsum3, rec2, total;
 };
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -143,7 +143,7 @@ struct hfs_ctx_s {
     // few instances without set plans: small1d_ok (complex64), cluster1d_ok (complex128)
     bool small = false, cluster = false;
     std::vector<int32_t> order;  // sorted position -> instance
-    std::vector<WorkItem> work;
+    std::vector<WorkItem> work[2];  // without and with the norm projection (default_ept): both on the device
     // schedule
     bool have_sched = false;
     SchedConst sc{};
@@ -224,7 +224,7 @@ Layout make_layout(const hfs_ctx_s *c, int64_t chunk)
     L.tdev = take(sizeof(double));
     L.inst = take(sizeof(DevInst) * c->count);
     L.order = take(sizeof(int32_t) * c->count);
-    L.work = take(sizeof(WorkItem) * std::max<int64_t>(c->count, 1));
+    for (auto &w : L.work) w = take(sizeof(WorkItem) * std::max<int64_t>(c->count, 1));
     L.twf = take(sizeof(float4) * kTwiddleTotal);
     L.twd = take(sizeof(cpx<double>) * kTwiddleTotal);
     L.twp = take(sizeof(float2) * kTwiddleTotal);
@@ -249,36 +249,42 @@ void build_worklist(hfs_ctx_s *c)
     std::iota(c->order.begin(), c->order.end(), 0);
     std::stable_sort(c->order.begin(), c->order.end(),
                      [&](int32_t x, int32_t y) { return c->inst[x].n[0] > c->inst[y].n[0]; });
-    c->work.clear();
     c->small = c->precision == HFS_C64 && small1d_ok(c->dinst.data(), c->count, c->elems, c->sm_count);
     c->cluster = c->precision == HFS_C128 && cluster1d_ok(c->dinst.data(), c->count, c->sm_count);
     for (auto &p : c->inst)
         if (c->plan_set[size_class(p.n[0])]) c->small = c->cluster = false;
     const bool fp64 = c->precision == HFS_C128, mixed = c->inst[c->order[0]].n[0] != c->inst[c->order[c->count - 1]].n[0];
-    int64_t i = 0;
-    while (i < c->count) {
-        const int n = c->inst[c->order[i]].n[0];
-        const bool set = c->plan_set[size_class(n)], alt = set && c->alt[size_class(n)];
-        const int e = set ? c->ept[size_class(n)] : default_ept(n, c->elems, mixed, c->norm_projection, c->sm_count, fp64);
-        const int per = kCtaThreads / (n / e);
-        int64_t j = i;
-        while (j < c->count && j - i < per && c->inst[c->order[j]].n[0] == n) ++j;
-        WorkItem w;
-        w.first = (int32_t)i;
-        w.count = (int32_t)(j - i);
-        w.plan = plan_id(n, e, alt);
-        w.diag = plan_id(n, set ? e : 16, alt);
-        c->work.push_back(w);
-        i = j;
+    for (int proj = 0; proj < 2; ++proj) {
+        c->work[proj].clear();
+        int64_t i = 0;
+        while (i < c->count) {
+            const int n = c->inst[c->order[i]].n[0];
+            const bool set = c->plan_set[size_class(n)], alt = set && c->alt[size_class(n)];
+            const int e = set ? c->ept[size_class(n)] : default_ept(n, c->elems, mixed, proj, c->sm_count, fp64);
+            const int per = kCtaThreads / (n / e);
+            int64_t j = i;
+            while (j < c->count && j - i < per && c->inst[c->order[j]].n[0] == n) ++j;
+            WorkItem w;
+            w.first = (int32_t)i;
+            w.count = (int32_t)(j - i);
+            w.plan = plan_id(n, e, alt);
+            w.diag = plan_id(n, set ? e : 16, alt);
+            c->work[proj].push_back(w);
+            i = j;
+        }
     }
 }
+
+const std::vector<WorkItem> &worklist(const hfs_ctx_s *c) { return c->work[c->norm_projection ? 1 : 0]; }
+WorkItem *worklist_dev(hfs_ctx_s *c) { return wptr<WorkItem>(c, c->lay.work[c->norm_projection ? 1 : 0]); }
 
 int upload_tables(hfs_ctx_s *c)
 {
     CK(cudaMemcpyAsync(wptr<void>(c, c->lay.order), c->order.data(), sizeof(int32_t) * c->count,
                        cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(wptr<void>(c, c->lay.work), c->work.data(), sizeof(WorkItem) * c->work.size(),
-                       cudaMemcpyHostToDevice, c->stream));
+    for (int proj = 0; proj < 2; ++proj)
+        CK(cudaMemcpyAsync(wptr<void>(c, c->lay.work[proj]), c->work[proj].data(), sizeof(WorkItem) * c->work[proj].size(),
+                           cudaMemcpyHostToDevice, c->stream));
     return HFS_OK;
 }
 
@@ -365,7 +371,7 @@ int check_validity(const hfs_ctx_s *c, int64_t nsteps)
 // the work list holds a plan of the wide set
 bool worklist_wide(const hfs_ctx_s *c)
 {
-    for (const WorkItem &w : c->work)
+    for (const WorkItem &w : worklist(c))
         if (plan_is_wide(w.plan)) return true;
     return false;
 }
@@ -377,7 +383,7 @@ int step_grid(const hfs_ctx_s *c, bool wide)
     const bool fp64 = c->precision == HFS_C128;
     const int fit = step1d_ctas_per_sm(fp64, c->variant, wide);
     const int per_sm = c->ctas_per_sm > 0 ? std::min(c->ctas_per_sm, fit) : fit;
-    return std::max(1, std::min<int>((int)c->work.size(), c->sm_count * per_sm));
+    return std::max(1, std::min<int>((int)worklist(c).size(), c->sm_count * per_sm));
 }
 
 // enqueue nsteps steps (no graph logic); work list already uploaded; rp:
@@ -430,8 +436,8 @@ int enqueue_steps(hfs_ctx_s *c, int64_t nsteps, const ReusePlan &rp = ReusePlan(
             a.psi = c->psi;
             a.inst = dinst;
             a.order = wptr<int32_t>(c, c->lay.order);
-            a.work = wptr<WorkItem>(c, c->lay.work);
-            a.nwork = (int32_t)c->work.size();
+            a.work = worklist_dev(c);
+            a.nwork = (int32_t)worklist(c).size();
             a.rec = rec_now;
             a.nrec = nstage + 1;
             a.tw = fp64 ? wptr<void>(c, c->lay.twd) : wptr<void>(c, c->lay.twf);
@@ -758,15 +764,6 @@ int hfs_set_norm_projection(hfs_ctx_t c, int enable)
     if (c->dim == 3 && c->inst[0].n[0] != 128) return HFS_ERR_UNSUPPORTED;
     c->norm_projection = enable != 0;
     drop_graphs(c);
-    if (c->dim == 1) {  // default plans depend on it
-        const std::vector<WorkItem> old = c->work;
-        build_worklist(c);
-        const bool same = old.size() == c->work.size() &&
-                          std::equal(old.begin(), old.end(), c->work.begin(), [](const WorkItem &x, const WorkItem &y) {
-                              return x.first == y.first && x.count == y.count && x.plan == y.plan && x.diag == y.diag;
-                          });
-        if (c->work_base && !same) return upload_tables(c);
-    }
     return HFS_OK;
 }
 
@@ -914,14 +911,14 @@ static int run_diag(hfs_ctx_s *c, bool energy)
         a.psi = c->psi;
         a.inst = wptr<DevInst>(c, c->lay.inst);
         a.order = wptr<int32_t>(c, c->lay.order);
-        a.work = wptr<WorkItem>(c, c->lay.work);
-        a.nwork = (int32_t)c->work.size();
+        a.work = worklist_dev(c);
+        a.nwork = (int32_t)worklist(c).size();
         a.tw = fp64 ? wptr<void>(c, c->lay.twd) : wptr<void>(c, c->lay.twf);
         a.t_dev = wptr<double>(c, c->lay.tdev);
         a.out = dout;
         a.pre = wptr<StageFGE>(c, c->lay.fge);  // free between calls
         a.count = c->count;
-        for (const WorkItem &w : c->work) a.ept[w.diag / kPlanCodes] = plan_ept(w.diag);
+        for (const WorkItem &w : worklist(c)) a.ept[w.diag / kPlanCodes] = plan_ept(w.diag);
         CK(launch_diag1d(fp64, energy, a, c->sm_count, c->stream));
     } else {
         Diag3DArgs a{};
