@@ -250,8 +250,9 @@ int hfs_sync_status(hfs_ctx_t ctx);
  * 4 for n <= 1024), | HFS_PLAN_ALT_ORDER for the alternative order of the
  * Stockham radices with 16 values per thread (radix 8 throughout at n = 4096,
  * the small radix first otherwise).  4 values per thread and the alternative
- * order are complex64 only.  Affects later hfs_step calls; a grid size whose
- * plan was not set takes one by the batch's sizes and its number of points.
+ * order are complex64 only.  Affects later hfs_step calls.  Without a set
+ * plan: 16 values per thread (complex64 without the norm projection 8 at n =
+ * 512 and 2048), or, for few instances, kernels of their own.
  * Errors: HFS_ERR_UNSUPPORTED. */
 #define HFS_PLAN_ALT_ORDER 0x100
 int hfs_set_plan(hfs_ctx_t ctx, int n, int plan);
@@ -309,7 +310,7 @@ int hfs_last_step_kernel_ms(hfs_ctx_t ctx, float *ms);
  * flow and built-in composition (HFS_COMP_CUSTOM is not accepted), on the
  * given stream (NULL: legacy default stream).  Results equal, bit for bit,
  * those of hfs_step() with a 16-step schedule chunk and the context's
- * defaults (plans chosen by the batch's sizes, norm projection off).
+ * defaults (no plan set, norm projection off).
  *
  * No device memory is allocated or freed: all scratch lives in one
  * file-scope __device__ array of HFS_NOALLOC_SCRATCH_BYTES that every GPU

@@ -73,21 +73,27 @@ int composition_fixed(int comp, double *a, double *b, int *m)
 }
 
 // Values per thread where no plan was set (batches that small1d_ok and
-// cluster1d_ok leave).  FP32 with the norm projection (plain twiddles): 16; 8
-// measured 1 to 5 % slower at 300 to 2000 instances, and rounds in one more pass.
-// FP32 without it: 8, on twice the threads, while these make at most two
-// 256-thread CTAs an SM (608 instances of 1024 points 4.05 against 4.78 us a step,
-// 1216 of them 7.7 against 6.7), at 512 points (three radix-8 passes; 3000
-// instances, 50 steps: 429 against 522 us) and for the sizes up to 1024 of a mixed
-// batch: their shorter, more numerous warps fill the gaps that the long
-// transforms' exchanges leave (4096 instances of 128 ... 4096 points, 60 steps:
-// 2.37 -> 2.20 ms).  FP64: 8 until the FP64 pipe has eight warps an SM.
-int default_ept(int n, int64_t points, bool mixed, bool proj, int sms, bool fp64)
+// cluster1d_ok leave): 16, or 8 on twice the threads where that is faster and ends no
+// further from 64 bits, which is so without the norm projection (compensated
+// twiddles) at 512 points (8 8 8 against 16 16 2: errors of 100 steps 1.416e-6 and
+// 1.420e-6; 200 instances, 50 steps: 201 -> 122 us, 3000: 516 -> 438 us) and 2048 (8 8
+// 8 4 against 16 16 8: 1.565e-6 and 1.575e-6; 300: 294 -> 237 us, 3000: 2134 -> 2029
+// us).  The other sizes take a pass more with 8: 1 to 3 % further off.  Under the
+// projection, with plain twiddles, 8 is 7 % further off; in FP64 12 to 20 % at 512 and
+// 1024 points, and no faster than 16 in small work items.
+int default_ept(int n, bool fp64, bool proj) { return !fp64 && !proj && (n == 512 || n == 2048) ? 8 : 16; }
+
+// Instances of a work item whose teams have `team` threads; warps: of the whole
+// batch.  A CTA takes 256 threads of them.  FP64: no more than give every SM its
+// share, but four warps, one for each quarter of the SM and its FP64 unit, since warps
+// without an instance leave at once (200 instances of 1024 points, 10 steps: 50 full
+// CTAs 1424 us, 100 of two instances 730 us).  FP32 warps without an instance run along.
+int item_instances(int team, int64_t warps, int sms, bool fp64)
 {
-    if (!fp64 && proj) return 16;
-    if (n <= 2048 && points / 8 <= (int64_t)sms * kCtaThreads * (fp64 ? 1 : 2)) return 8;
-    if (!fp64 && n <= 1024 && (mixed || n == 512)) return 8;
-    return 16;
+    const int full = kCtaThreads / team;
+    if (!fp64) return full;
+    const int64_t share = std::max<int64_t>(4, (warps + sms - 1) / sms);
+    return (int)std::min<int64_t>(full, (share * 32 + team - 1) / team);
 }
 
 // upper bound of omega over [t0, t1] for the validity check
@@ -253,15 +259,17 @@ void build_worklist(hfs_ctx_s *c)
     c->cluster = c->precision == HFS_C128 && cluster1d_ok(c->dinst.data(), c->count, c->sm_count);
     for (auto &p : c->inst)
         if (c->plan_set[size_class(p.n[0])]) c->small = c->cluster = false;
-    const bool fp64 = c->precision == HFS_C128, mixed = c->inst[c->order[0]].n[0] != c->inst[c->order[c->count - 1]].n[0];
+    const bool fp64 = c->precision == HFS_C128;
     for (int proj = 0; proj < 2; ++proj) {
+        auto ept = [&](int n) { return c->plan_set[size_class(n)] ? c->ept[size_class(n)] : default_ept(n, fp64, proj); };
+        int64_t threads = 0;
+        for (auto &p : c->inst) threads += p.n[0] / ept(p.n[0]);
         c->work[proj].clear();
         int64_t i = 0;
         while (i < c->count) {
-            const int n = c->inst[c->order[i]].n[0];
+            const int n = c->inst[c->order[i]].n[0], e = ept(n);
             const bool set = c->plan_set[size_class(n)], alt = set && c->alt[size_class(n)];
-            const int e = set ? c->ept[size_class(n)] : default_ept(n, c->elems, mixed, proj, c->sm_count, fp64);
-            const int per = kCtaThreads / (n / e);
+            const int per = item_instances(n / e, (threads + 31) / 32, c->sm_count, fp64);
             int64_t j = i;
             while (j < c->count && j - i < per && c->inst[c->order[j]].n[0] == n) ++j;
             WorkItem w;

@@ -150,14 +150,15 @@ extern "C" int hfs_step1d_noalloc(void *psi, int precision, const hfs_instance *
     const bool fp64 = precision == HFS_C128;
     for (int64_t i = 0; i < count; ++i) t_order[i] = (int32_t)i;
     std::stable_sort(t_order, t_order + count, [](int32_t x, int32_t y) { return t_inst[x].n[0] > t_inst[y].n[0]; });
-    const bool mixed = t_inst[t_order[0]].n[0] != t_inst[t_order[count - 1]].n[0];
     const bool small = !fp64 && small1d_ok(t_inst, count, off, sms);
     const bool cluster = fp64 && cluster1d_ok(t_inst, count, sms);
+    int64_t threads = 0;
+    for (int64_t i = 0; i < count; ++i) threads += t_inst[i].n[0] / default_ept(t_inst[i].n[0], fp64, false);
     int32_t nwork = 0;
     for (int64_t i = 0; i < count;) {
         const int n = t_inst[t_order[i]].n[0];
-        const int e = default_ept(n, off, mixed, false, sms, fp64);
-        const int per = kCtaThreads / (n / e);
+        const int e = default_ept(n, fp64, false);
+        const int per = item_instances(n / e, (threads + 31) / 32, sms, fp64);
         int64_t j = i;
         while (j < count && j - i < per && t_inst[t_order[j]].n[0] == n) ++j;
         t_work[nwork].first = (int32_t)i;

@@ -117,10 +117,10 @@ cudaError_t launch_twiddles(void *tw_f, void *tw_d, cudaStream_t st);
 // the plain FP32 table (same layout, the FP64 value rounded to float2)
 cudaError_t launch_twiddles_plain(void *tw_p, cudaStream_t st);
 
-// values per thread of grid size n in a batch without a set plan: points is
-// the batch's total, mixed whether it holds more than one grid size, proj the
-// norm projection (hfs_api.cu)
-int default_ept(int n, int64_t points, bool mixed, bool proj, int sms, bool fp64);
+// work items (hfs_api.cu): values per thread of grid size n without a set plan, and
+// instances of one item
+int default_ept(int n, bool fp64, bool proj);
+int item_instances(int team, int64_t warps, int sms, bool fp64);
 
 // host helpers shared by the entry points (hfs_api.cu)
 int composition_fixed(int comp, double *a, double *b, int *m);

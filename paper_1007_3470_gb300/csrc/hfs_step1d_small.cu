@@ -115,14 +115,16 @@ __device__ __forceinline__ void small_item(const Step1DArgs &a, int idx, const R
     if (bad) atomicOr(a.status, (unsigned)ST_NONFINITE);
 }
 
-// 2048 and 4096 points: eight and sixteen values a thread, as in the batch kernel
-// (with four, 512 and 1024 threads of 64 registers, 4096 points took 11.8 us a
-// step; 4.5 here)
+// 2048 points: eight values a thread or, under the projection, sixteen; 4096:
+// sixteen, as default_ept for the batch kernel (with four, 512 and 1024 threads of 64
+// registers, 4096 points took 11.8 us a step; 4.5 here)
 template <int N, int E, bool PROJ, int VI>
 __device__ __forceinline__ void big_item(const Step1DArgs &a, int idx, const RecF *rec, cpx<float> *sm, float *vtab,
                                          float *slots)
 {
-    static_assert(N / E == kCtaThreads, "the whole CTA is the team");
+    constexpr int T = N / E;
+    static_assert(T <= kCtaThreads, "one CTA is the team");
+    if (threadIdx.x >= T) return;
     const DevInst &ip = a.inst[idx];
     const TeamParams<float> tp = team_params<float>(ip);
     cpx<float> *psi = reinterpret_cast<cpx<float> *>(a.psi) + ip.off;
@@ -130,7 +132,7 @@ __device__ __forceinline__ void big_item(const Step1DArgs &a, int idx, const Rec
     const int t = threadIdx.x;
     cpx<float> v[E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) v[e] = ld_state(psi + t + kCtaThreads * e, a.streaming);
+    for (int e = 0; e < E; ++e) v[e] = ld_state(psi + t + T * e, a.streaming);
     vi_table<N, E, VI>(vtab, t, tp);
     step_loop<float, VI, N, E, false, PROJ>(a, v, t, 0, true, idx, rec, tp, sm, tw, vtab, slots);
     bool bad = false;
@@ -140,7 +142,7 @@ __device__ __forceinline__ void big_item(const Step1DArgs &a, int idx, const Rec
     }
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        st_state(psi + t + kCtaThreads * e, v[e], a.streaming);
+        st_state(psi + t + T * e, v[e], a.streaming);
         bad |= !(isfinite(v[e].x) && isfinite(v[e].y));
     }
     if (bad) atomicOr(a.status, (unsigned)ST_NONFINITE);
@@ -180,7 +182,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) small1d_kernel(const Small1DAr
     case 1024: small_item<1024, PROJ>(a, idx, rec, sm, vtab, slots); break;
     default:
         if constexpr (BIG) {
-            if (a.inst[idx].n[0] == 2048) big_item<2048, 8, PROJ, VI>(a, idx, rec, sm, vtab, slots);
+            if (a.inst[idx].n[0] == 2048) big_item<2048, PROJ ? 16 : 8, PROJ, VI>(a, idx, rec, sm, vtab, slots);
             else big_item<4096, 16, PROJ, VI>(a, idx, rec, sm, vtab, slots);
         }
     }

@@ -15,8 +15,9 @@ def _error(case, seeds, plan=0):
     errors = []
     for seed in seeds:
         state = cases.prepare(case, seed)
-        if plan:
-            state["solver"].set_plan(case["nmin"], plan)
+        for n in (128, 256, 512, 1024, 2048, 4096):
+            if plan and case["nmin"] <= n <= case["nmax"]:
+                state["solver"].set_plan(n, plan)
         psi = cases.run(state)
         torch.cuda.synchronize()
         exact = cases.exact(case, seed)
@@ -32,7 +33,7 @@ def _cube(n, **kw):
 
 def _batch(n, count, **kw):
     from perf import cases
-    return cases._solve1d(count=count, nmin=n, nmax=n, **kw)
+    return cases._solve1d(**dict(dict(count=count, nmin=n, nmax=n), **kw))
 
 
 @pytest.mark.parametrize("n", [512, 2048])
