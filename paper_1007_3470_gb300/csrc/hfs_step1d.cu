@@ -151,40 +151,52 @@ __device__ __forceinline__ void norm_item(const Diag1DArgs &a, const WorkItem &i
     if (active && t == 0) a.out[2 * idx] = s * ip.dx[0];
 }
 
-// The potential's sum over a thread's points in FP64: eight FP64 instructions a
-// point, cos k x by c_{e+1} = 2 cos(k T dx) c_e - c_{e-1} (its error of some E^2
-// roundings is far below the transform's).  c2 = mu omega^2 / 2; g, sg = cos, sin
-// of k T dx.
-template <int N, int E>
-__device__ __forceinline__ double potential_fp64(const DevInst &ip, const cpx<double> (&v)[E], int t, double c2, double g, double sg)
+// an integer as a double: behind the exponent of 2^52, one FP64 addition
+__device__ __forceinline__ double int64_of(int m)
 {
-    constexpr int T = N / E;
-    const double hs = 0.5 * ip.sigma, step = T * ip.dx[0];
-    const int kind = ip.eps != 0.0 ? ip.vi_kind : HFS_VI_NONE;
-    double x = ip.xc[0] + (double)(t - N / 2) * ip.dx[0];
-    double pot = 0.0, c = 0.0, cn = 0.0, f = 0.0;
-    if (kind == HFS_VI_COS) {
-        double sn, cs;
-        sincos(ip.vi_k * x, &sn, &cs);
-        f = 2.0 * g;
-        c = ip.eps * cs;
-        cn = ip.eps * (cs * g - sn * sg);
-    }
+    return __hiloint2double(0x43300000, (int)((unsigned)m ^ 0x80000000u)) - 4503601774854144.0;  // 2^52 + 2^31
+}
+
+// The potential's sum over a thread's points in FP64, nine FP64 instructions a point.
+// cos k x of point t + T e is that of the sum of k x_t and k T e dx.  The lanes of a
+// warp form the second ones' cosines and sines once, one e each, and pass them round:
+// two roundings a point whatever its e, where the recurrence c_{e+1} = 2 cos(k T dx)
+// c_e - c_{e-1} reached 1.7e-14 at e = 15 and a cosine for every point takes 45
+// instructions.  The points are read from memory, and once more for the transform: over
+// its registers the loop spilled.  c2 = mu omega^2 / 2.  Every lane of a warp calls this.
+template <int N, int E>
+__device__ __forceinline__ double potential_fp64(const DevInst &ip, const cpx<double> *psi, bool active, int t, double c2)
+{
+    constexpr int T = N / E, GW = T < E ? T : E;  // lanes that share the E cosines: of one team
+    const double hs = 0.5 * ip.sigma, dx = ip.dx[0], xc = ip.xc[0];
+    const int kind = ip.eps != 0.0 ? ip.vi_kind : HFS_VI_NONE, lane = threadIdx.x & 31;
+    bool cosine = kind == HFS_VI_COS;
+    if constexpr (T < 32) cosine = __any_sync(0xffffffffu, cosine);
+    double ac = 0.0, as = 0.0, bc[E / GW], bs[E / GW];
+    if (cosine) {
+        sincos(ip.vi_k * fma(int64_of(t - N / 2), dx, xc), &as, &ac);
+        const double eps = kind == HFS_VI_COS ? ip.eps : 0.0;
+        ac *= eps;
+        as *= -eps;
 #pragma unroll
+        for (int j = 0; j < E / GW; ++j) sincos(ip.vi_k * (int64_of(T * ((lane & (GW - 1)) + GW * j)) * dx), &bs[j], &bc[j]);
+    }
+    double pot = 0.0;
+#pragma unroll 4
     for (int e = 0; e < E; ++e) {
-        const double vx = v[e].x, vy = v[e].y;
+        const cpx<double> v = active ? psi[t + T * e] : cpx<double>{0.0, 0.0};
+        const double vx = v.x, vy = v.y, x = fma(int64_of(t + T * e - N / 2), dx, xc);
         const double d = fma(vx, vx, vy * vy), xx = x * x;
         double w = fma(hs, d, c2 * xx);
-        if (kind == HFS_VI_COS) {
-            w += c;
-            const double next = fma(f, cn, -c);
-            c = cn;
-            cn = next;
-        } else if (kind == HFS_VI_X4) {
-            w = fma(ip.eps * xx, xx, w);
+        if (cosine) {
+            const int from = (lane & ~(GW - 1)) | (e & (GW - 1));
+            const bool second = e >= GW;
+            const double c = __shfl_sync(0xffffffffu, bc[second ? E / GW - 1 : 0], from);
+            const double sn = __shfl_sync(0xffffffffu, bs[second ? E / GW - 1 : 0], from);
+            w = fma(as, sn, fma(ac, c, w));
         }
+        if (kind == HFS_VI_X4) w = fma(ip.eps * xx, xx, w);
         pot = fma(w, d, pot);
-        x += step;
     }
     return pot;
 }
@@ -315,10 +327,10 @@ __device__ __forceinline__ void energy_item(const Diag1DArgs &a, const WorkItem 
             kin = fma(m * m, fma(vx, vx, vy * vy), kin);
         }
     } else {
-        const StageFGE pre = a.pre[idx];
+        const double c2 = a.pre[idx].f;
+        pot = potential_fp64<N, E>(ip, psi, active, t, c2);
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = active ? psi[t + T * e] : cpx<R>{R(0), R(0)};
-        if (active) pot = potential_fp64<N, E>(ip, v, t, pre.f, pre.g, pre.e);
         FftPlan<N, E, ALT>::template run<false, R, 1, true>(v, sm, t, tw, 1 + g);
 #pragma unroll
         for (int e = 0; e < E; ++e) {
@@ -331,9 +343,9 @@ __device__ __forceinline__ void energy_item(const Diag1DArgs &a, const WorkItem 
     if (active && t == 0) a.out[2 * idx + 1] = fma(kin, a.out[2 * idx + 1], pot) * ip.dx[0];
 }
 
-// What every thread of an instance needs, once per instance: mu omega^2 / 2, cos,
-// sin of k T dx and the kinetic factor (with the law's sine and this sincos in
-// every thread the two calls took 0.34 ms); for an FP32 state in pairs.  One
+// What every thread of an instance needs, once per instance: mu omega^2 / 2 and the
+// kinetic factor, for an FP32 state cos, sin of k T dx as well, all in pairs (with the
+// law's sine and this sincos in every thread the two calls took 0.34 ms).  One
 // thread per instance: a CTA per work item left most lanes idle (16 us for 4096
 // instances, 11 us now, the latency of one thread).  The energy's slots of out
 // hold the kinetic factor and, for an FP32 state, sigma / 2 until it is written.
@@ -346,15 +358,13 @@ template <typename R> __global__ void energy_pre_kernel(const Diag1DArgs a)
     const double ku = 2.0 * 3.14159265358979323846 / ip.len[0];
     a.out[2 * idx + 1] = ku * ku / n / (2.0 * ip.mu);
     const double c2 = 0.5 * ip.mu * law_omega2(ip, *a.t_dev);
-    double sn, cs;
-    sincos(ip.vi_k * (ip.dx[0] * (n / a.ept[size_class(n)])), &sn, &cs);
     if constexpr (sizeof(R) == 8) {
         StageFGE r{};
         r.f = c2;
-        r.g = cs;
-        r.e = sn;
         a.pre[idx] = r;
     } else {
+        double sn, cs;
+        sincos(ip.vi_k * (ip.dx[0] * (n / a.ept[size_class(n)])), &sn, &cs);
         const double dx = ip.dx[0], d2 = dx * dx, ca = c2 * d2, cb = ip.eps * d2 * d2, r = ip.xc[0] / dx;
         const bool cosine = ip.vi_kind_eff == HFS_VI_COS;
         // zero, or within 1e-12 .. 1e8: with |m + r| <= 1e5 and |psi|^2 <= 1e6 no
