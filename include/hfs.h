@@ -267,9 +267,11 @@ int hfs_set_occupancy(hfs_ctx_t ctx, int ctas_per_sm);
  * over the grid sizes present, each trying every
  * admissible plan of that size (16, 8, 4 values per thread, the alternative
  * radix order) with the others fixed, keeping the fastest batch time; then
- * one CTA per SM against as many as fit.  Overwrites the state: call before
+ * one CTA per SM against as many as fit.  Few instances keep their own kernels
+ * and no plan is set unless a plan is faster.  Overwrites the state: call before
  * hfs_set_psi.  best_plans[6] (host, may be NULL) receives the chosen plan
- * (as for hfs_set_plan) for n = 128 ... 4096, 0 where the size is absent. */
+ * (as for hfs_set_plan; 16 where none is set) for n = 128 ... 4096, 0 where the
+ * size is absent. */
 int hfs_autotune(hfs_ctx_t ctx, int trial_steps, int32_t *best_plans);
 
 /* hfs_autotune with a persistent cache: the JSON file at `path` holds tuned

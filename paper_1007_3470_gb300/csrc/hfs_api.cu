@@ -1035,11 +1035,23 @@ int time_worklist(hfs_ctx_s *c, int64_t steps, cudaEvent_t e0, cudaEvent_t e1, f
     return HFS_OK;
 }
 
+// back to the plans of a context that has none set
+void clear_plans(hfs_ctx_s *c)
+{
+    for (int k = 0; k < kNumSizes; ++k) {
+        c->ept[k] = 16;
+        c->alt[k] = c->plan_set[k] = false;
+    }
+}
+
 // The search of hfs_autotune (see include/hfs.h): coordinate descent over
 // the grid sizes present, every candidate timed on the WHOLE batch (a size
 // class alone under-fills the GPU and favours plans with more, smaller
 // teams; a wide plan anywhere also moves the launch to the wide kernel),
-// two rounds; then one CTA per SM against as many as fit.
+// two rounds; then one CTA per SM against as many as fit.  Few instances have
+// kernels of their own that no set plan runs; they stay, with no plan set, unless the
+// best plans are faster (one instance of 1024 points: complex64 14.6 us a step
+// there, 31 with plans; complex128 20 and 38).
 int autotune(hfs_ctx_s *c, int trial_steps, float *best_total)
 {
     const int64_t steps = std::min<int64_t>(trial_steps, c->chunk);
@@ -1054,7 +1066,16 @@ int autotune(hfs_ctx_s *c, int trial_steps, float *best_total)
     CK(cudaEventCreate(&e1));
     const bool fp32 = c->precision == HFS_C64;
     int s = HFS_OK;
-    float total = INFINITY;
+    float total = INFINITY, few = INFINITY;
+    const int ctas_before = c->ctas_per_sm;
+    int ept[kNumSizes];
+    bool alt[kNumSizes], set[kNumSizes];
+    std::copy(c->ept, c->ept + kNumSizes, ept);
+    std::copy(c->alt, c->alt + kNumSizes, alt);
+    std::copy(c->plan_set, c->plan_set + kNumSizes, set);
+    clear_plans(c);
+    build_worklist(c);
+    if (c->small || c->cluster) s = time_worklist(c, steps, e0, e1, &few);
     // start point: 8 values per thread up to n = 1024 (several instances per
     // CTA), 16 above; each size's plan moves the batch time by about 1 %,
     // so the descent is sensitive to where it starts
@@ -1064,7 +1085,7 @@ int autotune(hfs_ctx_s *c, int trial_steps, float *best_total)
         c->plan_set[k] = true;
     }
     build_worklist(c);
-    s = time_worklist(c, steps, e0, e1, &total);
+    if (!s) s = time_worklist(c, steps, e0, e1, &total);
     const int cand[4] = {16, 8, 16 | HFS_PLAN_ALT_ORDER, 4};
     for (int round = 0; round < 2 && !s; ++round) {
         for (int k = 0; k < kNumSizes && !s; ++k) {
@@ -1100,6 +1121,16 @@ int autotune(hfs_ctx_s *c, int trial_steps, float *best_total)
         s = time_worklist(c, steps, e0, e1, &ms);
         if (!s && ms < total) total = ms;
         else c->ctas_per_sm = keep;
+    }
+    if (s) {  // as before the call
+        std::copy(ept, ept + kNumSizes, c->ept);
+        std::copy(alt, alt + kNumSizes, c->alt);
+        std::copy(set, set + kNumSizes, c->plan_set);
+        c->ctas_per_sm = ctas_before;
+    } else if (few <= total) {
+        clear_plans(c);
+        c->ctas_per_sm = ctas_before;
+        total = few;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1169,6 +1200,7 @@ struct CacheEntry {
     int plans[kNumSizes];
     int ctas_per_sm;
     double ms;
+    bool few;  // the kernels of few instances, no plan set
 };
 
 bool read_file(const char *path, std::string &out)
@@ -1199,8 +1231,11 @@ std::vector<CacheEntry> parse_cache(const std::string &text)
         if (pl == std::string::npos || (nl != std::string::npos && pl > nl)) continue;
         if (sscanf(text.c_str() + pl, "\"plans\": [%d, %d, %d, %d, %d, %d], \"ctas_per_sm\": %d, \"ms\": %lf",
                    &e.plans[0], &e.plans[1], &e.plans[2], &e.plans[3], &e.plans[4], &e.plans[5], &e.ctas_per_sm,
-                   &e.ms) == 8)
+                   &e.ms) == 8) {
+            const size_t few = text.find("\"few\": 1", pl);
+            e.few = few != std::string::npos && (nl == std::string::npos || few < nl);
             v.push_back(e);
+        }
         pos = end;
     }
     return v;
@@ -1214,9 +1249,9 @@ bool write_cache(const char *path, const std::vector<CacheEntry> &v)
     fprintf(f, "{\"hfs_tuned_plans\": 1, \"entries\": [\n");
     for (size_t i = 0; i < v.size(); ++i) {
         const CacheEntry &e = v[i];
-        fprintf(f, "  {\"key\": \"%s\", \"plans\": [%d, %d, %d, %d, %d, %d], \"ctas_per_sm\": %d, \"ms\": %.4f}%s\n",
+        fprintf(f, "  {\"key\": \"%s\", \"plans\": [%d, %d, %d, %d, %d, %d], \"ctas_per_sm\": %d, \"ms\": %.4f%s}%s\n",
                 e.key.c_str(), e.plans[0], e.plans[1], e.plans[2], e.plans[3], e.plans[4], e.plans[5], e.ctas_per_sm,
-                e.ms, i + 1 < v.size() ? "," : "");
+                e.ms, e.few ? ", \"few\": 1" : "", i + 1 < v.size() ? "," : "");
     }
     fprintf(f, "]}\n");
     const bool ok = fclose(f) == 0;
@@ -1239,7 +1274,13 @@ int hfs_autotune_cache(hfs_ctx_t c, const char *path, int trial_steps, int32_t *
     if (read_file(path, text)) entries = parse_cache(text);
     for (const CacheEntry &e : entries) {
         if (e.key != key) continue;
-        for (int k = 0; k < kNumSizes; ++k) {
+        if (e.few) {
+            clear_plans(c);
+            build_worklist(c);
+            s = upload_tables(c);
+            if (s) return s;
+        }
+        for (int k = 0; k < kNumSizes && !e.few; ++k) {
             if (!e.plans[k]) continue;
             s = hfs_set_plan(c, 128 << k, e.plans[k]);
             if (s) return s;
@@ -1269,6 +1310,7 @@ int hfs_autotune_cache(hfs_ctx_t c, const char *path, int trial_steps, int32_t *
     for (int k = 0; k < kNumSizes; ++k) e.plans[k] = present[k] ? encode_plan(c, k) : 0;
     e.ctas_per_sm = c->ctas_per_sm;
     e.ms = total;
+    e.few = c->small || c->cluster;
     bool replaced = false;
     for (CacheEntry &o : entries)
         if (o.key == key) {
