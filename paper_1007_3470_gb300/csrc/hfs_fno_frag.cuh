@@ -12,7 +12,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
+#include "hfs_resident.h"
 
 namespace hfs {
 namespace fno {
@@ -251,38 +251,26 @@ inline cudaError_t launch_k(void (*kernel)(P...), dim3 grid, int threads, size_t
     return cudaLaunchKernelEx(&cfg, kernel, a...);
 }
 
-// CTAs of a persistent grid: as many as fit.  Asked once for a kernel, its
-// shared memory and a device; the slot is the launch site's own, and a race of
-// two threads on it only asks twice.  Every kernel is allowed the most shared
-// memory that a CTA may have (none has static arrays), whatever its launch
-// takes, so that models of different sizes do not undo each other's setting.
+// CTAs of a persistent grid: as many as fit (remembered, see ResidentSlot).  Every
+// kernel is allowed the most shared memory that a CTA may have (none has static
+// arrays), whatever its launch takes, so that models of different sizes do not undo
+// each other's setting.
 constexpr int kMaxSmem = 227 * 1024;
-struct ResidentSlot {
-    std::atomic<uint64_t> dev[16];  // (shared memory + 1) << 24 | CTAs
-};
 template <typename K>
 inline cudaError_t resident_ctas(ResidentSlot &slot, K kernel, int threads, size_t smem, int *ctas)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    const bool keep = dev >= 0 && dev < 16;
-    if (keep) {
-        const uint64_t v = slot.dev[dev].load(std::memory_order_relaxed);
-        if ((v >> 24) == (uint64_t)smem + 1) {
-            *ctas = (int)(v & 0xffffff);
-            return cudaSuccess;
-        }
-    }
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-    int sms = 0, per = 0;
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
-    if (e == cudaSuccess && per < 1) e = cudaErrorInvalidConfiguration;
-    if (e != cudaSuccess) return e;
-    *ctas = sms * per;
-    if (keep) slot.dev[dev].store(((uint64_t)smem + 1) << 24 | (uint64_t)*ctas, std::memory_order_relaxed);
-    return cudaSuccess;
+    return (cudaError_t)slot.get(dev, threads, smem, [&](int *n) -> int {
+        int sms = 0, per = 0;
+        cudaError_t q = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        if (q == cudaSuccess) q = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (q == cudaSuccess) q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
+        if (q == cudaSuccess && per < 1) q = cudaErrorInvalidConfiguration;
+        *n = sms * per;
+        return (int)q;
+    }, ctas);
 }
 
 __host__ __device__ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v >> 1); }
