@@ -156,8 +156,11 @@ __device__ __forceinline__ unsigned pack2(float lo, float hi)
 // so the value v differs from gelu_f(z), whose own error is below 1.5e-7 |z|,
 // by less than d = 6e-7 |z|.  Where v - d and v + d round to the same BF16
 // number, so does gelu_f(z); in the other cases (1 in 1000 values to 7000,
-// and every z below -5) the accurate function decides.  (Checked over all 2^32
-// values of z: equal but for z = -0, where this gives +0.)
+// and every z below -5) the accurate function decides.  Over all 2^32 values of z
+// the result is equal but for z = -0, where this gives +0 (test_gelu_over_all_inputs).
+// The time depends on the values: a group with one below -5 takes both paths; 4096
+// samples whose every pre-activation is near -8 take 1.18 ms, 0.89 with the usual ones
+// (3.52 ms GEMM by GEMM, either way).
 static __device__ __noinline__ uint2 gelu4_accurate(float a, float b, float c, float d)
 {
     return make_uint2(pack2(gelu_f(a), gelu_f(b)), pack2(gelu_f(c), gelu_f(d)));

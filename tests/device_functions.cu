@@ -3,6 +3,7 @@
 #include <cstdio>
 #include <cstring>
 
+#include "hfs_fno_frag.cuh"
 #include "hfs_phase.cuh"
 
 using namespace hfs;
@@ -34,12 +35,30 @@ __global__ void turns_modulus(double *worst)
     atomic_max(worst, e >= 0.0 ? e : 1e300);
 }
 
+// gelu4 against bf16(gelu_f) over all 2^32 values of z, in each of its four places:
+// values that differ
+__global__ void gelu_differences(double *count)
+{
+    const unsigned long long n = gridDim.x * (unsigned long long)blockDim.x;
+    unsigned long long bad = 0;
+    for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < (1ull << 32); i += n) {
+        const float z = __uint_as_float((unsigned)i), o = 0.5f;
+        const unsigned ref = fno::pack2(fno::gelu_f(z), fno::gelu_f(o));
+        const uint2 a = fno::gelu4(z, o, 1.0f, 2.0f), b = fno::gelu4(1.0f, 2.0f, z, o);
+        const uint2 c = fno::gelu4(o, z, 1.0f, 2.0f), d = fno::gelu4(1.0f, 2.0f, o, z);
+        const unsigned swapped = ref << 16 | ref >> 16;
+        bad += a.x != ref || b.y != ref || c.x != swapped || d.y != swapped;
+    }
+    atomicAdd(count, (double)bad);
+}
+
 int main(int, char **argv)
 {
     double *d = nullptr, h = 0.0;
     if (cudaMalloc(&d, 8) != cudaSuccess || cudaMemset(d, 0, 8) != cudaSuccess) return 1;
     if (!strcmp(argv[1], "turns_error")) turns_error<<<4096, 256>>>(d);
     else if (!strcmp(argv[1], "turns_modulus")) turns_modulus<<<4096, 256>>>(d);
+    else if (!strcmp(argv[1], "gelu_differences")) gelu_differences<<<1520, 256>>>(d);
     else return 1;
     if (cudaMemcpy(&h, d, 8, cudaMemcpyDeviceToHost) != cudaSuccess) return 1;
     printf("%.17g\n", h);

@@ -56,3 +56,8 @@ def test_fp64_state_of_an_absurd_interaction_keeps_its_norm(plan, sigma):
     assert s.status() == hfs.HFS_OK
     assert np.all(np.abs(s.norm() / before - 1) <= 1e-14)
     s.close()
+
+
+def test_gelu_over_all_inputs(check):
+    """Equal to the accurate function rounded to BF16 but for -0, where it gives +0."""
+    assert check("gelu_differences") == 1
