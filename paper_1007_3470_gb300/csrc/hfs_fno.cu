@@ -721,11 +721,16 @@ int hfs_fno_forward(hfs_fno_t f, const float *x, float *y, int32_t batch)
     if (!f->params || !f->work) return HFS_ERR_NOT_READY;
     if (batch < 1 || batch > f->max_batch) return HFS_ERR_INVALID_ARG;
     (void)cudaGetLastError();
-    if (use_fused(f)) return forward_fused(f, x, batch, y, nullptr, false);
-    int s = forward(f, x, batch);
+    const uintptr_t xa = (uintptr_t)x, ya = (uintptr_t)y;
+    const size_t xn = 4 * (size_t)batch * f->cfg.grid * f->cfg.in_ch, yn = 4 * (size_t)batch * f->cfg.grid * f->cfg.out_ch;
+    // of a model with one layer the launch that writes y reads x: where they overlap,
+    // y comes through the workspace, as it does GEMM by GEMM
+    const bool apart = f->cfg.layers > 1 || xa + xn <= ya || ya + yn <= xa;
+    const bool fused = use_fused(f);
+    if (fused && apart) return forward_fused(f, x, batch, y, nullptr, false);
+    int s = fused ? forward_fused(f, x, batch, at<float>(f, f->off.O), nullptr, false) : forward(f, x, batch);
     if (s) return s;
-    FCK(cudaMemcpyAsync(y, at<float>(f, f->off.O), 4 * (size_t)batch * f->cfg.grid * f->cfg.out_ch,
-                        cudaMemcpyDeviceToDevice, f->stream));
+    FCK(cudaMemcpyAsync(y, at<float>(f, f->off.O), yn, cudaMemcpyDeviceToDevice, f->stream));
     return HFS_OK;
 }
 
