@@ -736,6 +736,7 @@ static cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
     return cudaLaunchKernelEx(&cfg, kernel, a, j);
 }
 
+// the line passes: FP64, and FP32 with the tensor-core z-pass at 64^3
 template <typename R, int N> static cudaError_t run3d(const Step3DArgs &a, cudaStream_t st)
 {
     using GEO = LineGeo<R, N>;
@@ -748,21 +749,17 @@ template <typename R, int N> static cudaError_t run3d(const Step3DArgs &a, cudaS
         if ((e = allow_smem(xpass3d<R, N, X_INV | X_PHASE>, xs)) != cudaSuccess) return e;
         if ((e = allow_smem(ypass3d<R, N, false>, ts)) != cudaSuccess) return e;
         if ((e = allow_smem(ypass3d<R, N, true>, ts)) != cudaSuccess) return e;
-        if ((e = allow_smem(zpass3d<R, N>, ts)) != cudaSuccess) return e;
-        if constexpr (sizeof(R) == 4 && (N == 64 || N == 128))
-            if ((e = allow_smem(zpass3d_tc<N>, zpass_tc_smem<N>())) != cudaSuccess) return e;
+        if constexpr (sizeof(R) == 4) e = allow_smem(zpass3d_tc<N>, zpass_tc_smem<N>());
+        else e = allow_smem(zpass3d<R, N>, ts);
+        if (e != cudaSuccess) return e;
         prepared = true;
     }
     const dim3 xg(N * N / GEO::G), tg(N / GEO::TX, N);
     xpass3d<R, N, X_PHASE | X_FWD><<<xg, GEO::THREADS, xs, st>>>(a, 0);
     ypass3d<R, N, false><<<tg, GEO::TT, ts, st>>>(a);
     for (int64_t j = 0; j < a.nstage; ++j) {
-        if constexpr (sizeof(R) == 4 && (N == 64 || N == 128)) {
-            if (a.dft_tc) zpass3d_tc<N><<<tg, GEO::TT, zpass_tc_smem<N>(), st>>>(a, j);
-            else zpass3d<R, N><<<tg, GEO::TT, ts, st>>>(a, j);
-        } else {
-            zpass3d<R, N><<<tg, GEO::TT, ts, st>>>(a, j);
-        }
+        if constexpr (sizeof(R) == 4) zpass3d_tc<N><<<tg, GEO::TT, zpass_tc_smem<N>(), st>>>(a, j);
+        else zpass3d<R, N><<<tg, GEO::TT, ts, st>>>(a, j);
         ypass3d<R, N, true><<<tg, GEO::TT, ts, st>>>(a);
         if (j + 1 < a.nstage) {
             xpass3d<R, N, X_INV | X_PHASE | X_FWD><<<xg, GEO::THREADS, xs, st>>>(a, j + 1);
