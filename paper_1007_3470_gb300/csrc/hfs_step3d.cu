@@ -487,8 +487,9 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane3d(const Step3DArgs a, 
 // with eight values a thread (n^2/8 threads hold a whole plane, one line
 // transform each at a time) and every launch programmatic.  Bound by latency:
 // the state lies in L2 and a pass is one chain of load, transforms and store.
-// Four line passes took 17.8 us a step at 64^3 and 17.8 us at 32^3 (27 us without
-// graph replay); these take 8.4 us and 4.3 us.
+// Four line passes took 17.8 us a step at 64^3 and 15.9 us at 32^3 (graph replay);
+// these take 8.3 us and 4.4 us.  States end 0.6 % further from 64 bits at 64^3 (8 8
+// against 16 4) and 1.5 % less far at 32^3.
 // ---------------------------------------------------------------------------
 template <int N> struct Cube {
     static constexpr int E = 8, T = N / E, ROW = smem_elems(N);
