@@ -174,12 +174,13 @@ __device__ __forceinline__ double potential_fp64(const DevInst &ip, const cpx<do
     if constexpr (T < 32) cosine = __any_sync(0xffffffffu, cosine);
     double ac = 0.0, as = 0.0, bc[E / GW], bs[E / GW];
     if (cosine) {
-        sincos(ip.vi_k * fma(int64_of(t - N / 2), dx, xc), &as, &ac);
-        const double eps = kind == HFS_VI_COS ? ip.eps : 0.0;
+        // a neighbour's lanes in a warp of several teams add zero
+        const double eps = kind == HFS_VI_COS ? ip.eps : 0.0, k = kind == HFS_VI_COS ? ip.vi_k : 0.0;
+        sincos(k * fma(int64_of(t - N / 2), dx, xc), &as, &ac);
         ac *= eps;
         as *= -eps;
 #pragma unroll
-        for (int j = 0; j < E / GW; ++j) sincos(ip.vi_k * (int64_of(T * ((lane & (GW - 1)) + GW * j)) * dx), &bs[j], &bc[j]);
+        for (int j = 0; j < E / GW; ++j) sincos(k * (int64_of(T * ((lane & (GW - 1)) + GW * j)) * dx), &bs[j], &bc[j]);
     }
     double pot = 0.0;
 #pragma unroll 4

@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
 def test_perturbation_energy(n, plan, step):
     """One point each of instances with eps = 1e6, everywhere in the box, k T dx =
     `step` (T threads hold points T apart; a recurrence over them is worst near 0 and
-    pi), other kinds between them.  eps cos(k x) is off by the rounding of k x as a sum
+    pi), other kinds, whose k is
+    not read, between them.  eps cos(k x) is off by the rounding of k x as a sum
     of two products, 2 2^-53 (|k x_t| + |k T e dx|) |sin k x|, and by 2^-53 times: 2 for
     each sine or cosine, 1 for each product, the sum of products and the sum of terms,
     8 in all.  The other terms are exact to 1e-14 of their size (12 passes of the
@@ -28,7 +29,7 @@ def test_perturbation_energy(n, plan, step):
     for i, j in enumerate(points + [0, n // 3, n - 1]):
         kind = W.VI_COS if i < len(points) else (W.VI_NONE, W.VI_X4, W.VI_NONE)[i - len(points)]
         insts.append(W.Instance(n=[n], a=[-half], b=[half], w0=1.0, eps=eps if kind == W.VI_COS else 1e-3, vi_kind=kind,
-                                vi_k=k, sigma=2.0))
+                                vi_k=k if kind == W.VI_COS else np.nan, sigma=2.0))
         psi = np.zeros(n, dtype=np.complex128)
         psi[j] = (0.6 - 0.8j) / np.sqrt(dx)
         psis.append(psi)
