@@ -56,9 +56,9 @@ def tune(solver, trial_steps):
 # DRAM bytes per launch of the fused step kernel (dram__bytes_read.sum +
 # dram__bytes_write.sum from one ncu capture of the same command, summarised in
 # profiles/), valid only while the kernel's sources hash to "src".
-STEP1D_TRAFFIC = {"src": "88d5e6598e9904c5",
-                  "batch_1d_4096x500_c64": 109323520 + 16402432,
-                  "batch_1d_65536x1_streaming": (727424512 + 646248960 + 727406080 + 643721728) // 2}
+STEP1D_TRAFFIC = {"src": "d93670f2d6929390",
+                  "batch_1d_4096x500_c64": 109324800 + 16421888,
+                  "batch_1d_65536x1_streaming": (727472128 + 647481344 + 727436032 + 644759552) // 2}
 STEP1D_SOURCES = ("hfs_step1d.cuh", "hfs_step1d.cu", "hfs_step1d_vicos.cu", "hfs_step1d_vix4.cu", "hfs_step1d_vinone.cu",
                   "hfs_step1d_wide.cu", "hfs_step1d_wide_vicos.cu", "hfs_step1d_wide_vix4.cu",
                   "hfs_step1d_wide_vinone.cu", "hfs_fft.cuh", "hfs_phase.cuh", "hfs_internal.cuh", "hfs_sched.h")
